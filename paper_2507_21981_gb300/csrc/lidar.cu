@@ -15,12 +15,8 @@
 // tree's quality follows the storage order: Z-ordered nodes (dgs_spatial_order) give compact
 // leaves.  Trees are never refitted per env: rays are moved into each node's frame instead.
 //
-// Tracing: one thread per ray, one warp per packet of 32 rays.  A round collects, over every
-// node of the ray's env, the K nearest hits whose (t*, id) key follows the last key
-// composited, in a sorted buffer in shared memory; the packet's traversal is front to back and skips
-// boxes outside every lane's [t_last, t of its K-th hit].  The round's hits are composited;
-// the next round resumes after the last of them, until the transmittance drops below t_min or
-// fewer than K hits were left.
+// Tracing: one warp per ray, its lanes testing 32 boxes or 32 Gaussians at a time (see
+// k_lidar_trace).
 #include <algorithm>
 
 #include "dgs_internal.cuh"
@@ -29,9 +25,6 @@ namespace dgs {
 namespace {
 
 constexpr int kLeaf = 8;             // Gaussians per leaf
-constexpr int kKbuf = 32;            // hits per round
-constexpr int kStack = 40;           // traversal stack (depth <= 31 levels + the far children)
-constexpr int kTraceThreads = 128;
 
 __device__ __forceinline__ float sigmoidf(float x) { return 1.f / (1.f + __expf(-x)); }
 
@@ -172,206 +165,319 @@ __device__ __forceinline__ float slab_enter(const float4 lo, const float4 hi, co
     return fmaxf(fmaxf(fminf(x0, x1), fminf(y0, y1)), fminf(z0, z1));
 }
 
-// Per lane, in dynamic shared memory (lane-interleaved: entry i of thread x at [i][x]): the
-// round's sorted hits as bits of t*, global id and alpha; (t bits, id) is the 64-bit order key.
-constexpr size_t kKbufBytes = (size_t)3 * kKbuf * kTraceThreads * sizeof(uint32_t);
+// Per-warp state in shared memory: the traversal stack (heap index, slot and entry distance of
+// every node still to visit) and the pending hits (bits of t*, global id, alpha), unsorted.
+constexpr int kRayWarps = 4;         // warps (rays in flight) per block
+constexpr int kStack = 256;          // 32 roots + 31 per expansion, at most 6 expansions deep: 218
+constexpr int kPend = 128;           // pending hits
+constexpr int kPendRegs = kPend / 32;
+constexpr int kKeep = 64;            // hits kept when the pending buffer is cut
+struct RayWarp {
+    uint32_t node[kStack], slot[kStack];
+    float enter[kStack];
+    uint32_t t[kPend], g[kPend];
+    float a[kPend];
+};
 
-// Warp = a packet of up to 32 rays (consecutive ray numbers: make them neighbours in the beam
-// pattern).  The packet walks each tree together on a warp-uniform stack: a box is descended
-// if it holds the interval of any lane's ray, the children in the order of the first such
-// lane's entry distances; records and boxes are read once per warp.  Each lane keeps its own
-// hit buffer, interval and compositing state, and rounds repeat while any lane is unfinished.
-// Lanes whose sensor differs in a slot's node take the tree in turns.  Warps are persistent:
-// each takes the next 32 rays from a counter until none are left, so that packets of very
-// different cost (rays grazing a surface, many rounds) do not leave SMs idle at the end.
-__global__ void __launch_bounds__(kTraceThreads) k_lidar_trace(const LidarTreeDev* __restrict__ trees,
-                                                               const LidarSlot* __restrict__ slots, int K,
-                                                               const float* __restrict__ dirs, int n_dirs,
-                                                               int64_t n_rays, LidarParams LP,
-                                                               float* __restrict__ out_d, float* __restrict__ out_a,
-                                                               uint32_t* __restrict__ err,
-                                                               unsigned long long* __restrict__ next_ray,
-                                                               unsigned long long n_packets, unsigned long long scramble) {
-    __shared__ int s_stack[kTraceThreads / 32][kStack];
-    extern __shared__ uint32_t s_kbuf[];
-    uint32_t* const kt = s_kbuf + threadIdx.x;                      // entry i at kt[i * kTraceThreads]
-    uint32_t* const kg = kt + kKbuf * kTraceThreads;
-    float* const ka = reinterpret_cast<float*>(kg + kKbuf * kTraceThreads);
-    const int lane = threadIdx.x & 31;
-    int* stk = s_stack[threadIdx.x >> 5];
+// A ray in a slot's node frame.
+struct NodeRay {
+    float o[3], d[3], id[3];
+};
+
+__device__ __forceinline__ NodeRay node_ray(const LidarSlot& S, const float (&ds)[3]) {
+    NodeRay r;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        r.o[a] = S.o[a];
+        r.d[a] = S.R[3 * a] * ds[0] + S.R[3 * a + 1] * ds[1] + S.R[3 * a + 2] * ds[2];
+        r.id[a] = 1.f / r.d[a];
+    }
+    return r;
+}
+
+// Pushes the lanes with `in` set onto the stack, nearest entry on top (ties by lane).
+__device__ __forceinline__ void push_sorted(RayWarp& W, int& sp, bool in, float enter, uint32_t node, uint32_t slot, int lane) {
+    const unsigned m = __ballot_sync(0xffffffffu, in);
+    int rank = 0;
+    for (unsigned rest = m; rest; rest &= rest - 1) {
+        const int src = __ffs(rest) - 1;
+        const float e = __shfl_sync(0xffffffffu, enter, src);
+        rank += e < enter || (e == enter && src < lane);
+    }
+    const int n = __popc(m);
+    if (in) {
+        const int at = sp + n - 1 - rank;
+        W.node[at] = node;
+        W.slot[at] = slot;
+        W.enter[at] = enter;
+    }
+    sp += n;
+    __syncwarp();
+}
+
+// The pending hits in registers, entry 32 q + lane in slot q (key ~0: none), and back.
+__device__ __forceinline__ void load_pending(const RayWarp& W, int cnt, int lane, uint64_t (&key)[kPendRegs], float (&al)[kPendRegs]) {
+#pragma unroll
+    for (int q = 0; q < kPendRegs; ++q) {
+        const int i = 32 * q + lane;
+        key[q] = i < cnt ? ((uint64_t)W.t[i] << 32) | W.g[i] : ~0ull;
+        al[q] = i < cnt ? W.a[i] : 0.f;
+    }
+    __syncwarp();
+}
+
+__device__ __forceinline__ int store_pending(RayWarp& W, int lane, const uint64_t (&key)[kPendRegs], const float (&al)[kPendRegs]) {
+    int cnt = 0;
+#pragma unroll
+    for (int q = 0; q < kPendRegs; ++q) {
+        const bool live = key[q] != ~0ull;
+        const unsigned m = __ballot_sync(0xffffffffu, live);
+        if (live) {
+            const int at = cnt + __popc(m & ((1u << lane) - 1u));
+            W.t[at] = (uint32_t)(key[q] >> 32);
+            W.g[at] = (uint32_t)key[q];
+            W.a[at] = al[q];
+        }
+        cnt += __popc(m);
+    }
+    __syncwarp();
+    return cnt;
+}
+
+// Composites the pending hits with t* < bound in (t*, id) order, one warp-wide minimum per hit,
+// and keeps the others.  Returns true when the transmittance ends the ray.
+__device__ __forceinline__ bool composite_pending(RayWarp& W, int& cnt, float bound, float t_min, int lane, float& T, float& D) {
+    uint64_t key[kPendRegs];
+    float al[kPendRegs];
+    load_pending(W, cnt, lane, key, al);
+    bool done = false;
     for (;;) {
-        unsigned long long pk = 0;
-        if (lane == 0) pk = atomicAdd(next_ray, 1ull);
-        pk = __shfl_sync(0xffffffffu, pk, 0);
-        if (pk >= n_packets) break;
-        // packets in a scrambled order (p -> p * scramble mod n_packets, a bijection): costly
-        // packets that are neighbours in ray order do not all start last
-        const unsigned long long base = (unsigned long long)((unsigned __int128)pk * scramble % n_packets) * 32ull;
-        const int64_t ray = (int64_t)base + lane;
-        const bool valid = ray < n_rays;
-        int s = 0, j = 0;
-        float ds[3] = {1.f, 0.f, 0.f};
-        if (valid) {
-            s = (int)(ray / n_dirs);
-            j = (int)(ray - (int64_t)s * n_dirs);
-            ds[0] = dirs[3 * j]; ds[1] = dirs[3 * j + 1]; ds[2] = dirs[3 * j + 2];
+        uint64_t mine = key[0];
+        float a = al[0];
+#pragma unroll
+        for (int q = 1; q < kPendRegs; ++q)
+            if (key[q] < mine) { mine = key[q]; a = al[q]; }
+        const uint32_t tb = __reduce_min_sync(0xffffffffu, (uint32_t)(mine >> 32));
+        if (tb == ~0u || !(__uint_as_float(tb) < bound)) break;
+        const uint32_t gb = __reduce_min_sync(0xffffffffu, (uint32_t)(mine >> 32) == tb ? (uint32_t)mine : ~0u);
+        const uint64_t best = ((uint64_t)tb << 32) | gb;
+        a = __shfl_sync(0xffffffffu, a, __ffs(__ballot_sync(0xffffffffu, mine == best)) - 1);
+        const float Tn = fmaf(-a, T, T);
+        if (Tn < t_min) { done = true; break; }
+        D = fmaf(a * T, __uint_as_float(tb), D);
+        T = Tn;
+#pragma unroll
+        for (int q = 0; q < kPendRegs; ++q)
+            if (key[q] == best) key[q] = ~0ull;
+    }
+    cnt = done ? 0 : store_pending(W, lane, key, al);
+    return done;
+}
+
+// Keeps the kKeep nearest of more pending hits; returns the key of the farthest kept (the kKeep-th
+// smallest, found bit by bit: the largest x with fewer than kKeep keys below it).
+__device__ __forceinline__ uint64_t cut_pending(RayWarp& W, int& cnt, int lane) {
+    uint64_t key[kPendRegs];
+    float al[kPendRegs];
+    load_pending(W, cnt, lane, key, al);
+    uint64_t x = 0;
+    for (int b = 63; b >= 0; --b) {
+        const uint64_t c = x | (1ull << b);
+        int below = 0;
+#pragma unroll
+        for (int q = 0; q < kPendRegs; ++q) below += __popc(__ballot_sync(0xffffffffu, key[q] < c));
+        if (below < kKeep) x = c;
+    }
+#pragma unroll
+    for (int q = 0; q < kPendRegs; ++q)
+        if (key[q] > x) key[q] = ~0ull;
+    cnt = store_pending(W, lane, key, al);
+    return x;
+}
+
+// Warp = one ray at a time; persistent warps take the next ray from a counter.  Beams of a
+// sensor are farther apart, at the distances where they hit, than the Gaussians are wide, so
+// neighbouring rays share few leaves: the 32 lanes work on one ray instead, 32 boxes or 32
+// Gaussians per step.
+//   expand   the 2^s (s <= 5) descendants of a node s levels down are consecutive in heap
+//            numbering: one box per lane, one coalesced load; those the ray's interval meets are
+//            pushed nearest on top.  The first expansion of a tree takes the levels that do not
+//            divide by five.
+//   leaves   up to four leaves on top of the stack, 8 lanes each: one Gaussian per lane; hits go
+//            to the pending buffer.
+//   flush    a hit is final once its t* lies before the entry of every node still on the stack;
+//            final hits are composited in (t*, id) order, so one traversal composites the whole
+//            ray and ends as soon as the transmittance does.
+// When the pending buffer fills with hits that are not final, the nearest kKeep stay, nodes and
+// hits beyond them are skipped, and another round resumes after them.  The trees of up to 32
+// slots share one stack; with more, a slot batch is traversed after the other and hits are
+// final at the end of the round only.
+// Bound by latency (boxes and records come from L2, one dependent load per step), which the 24
+// or more warps per SM hide.  Measured against a packet of 32 rays per warp with a 32-hit buffer
+// per lane, same outputs bit for bit: one sensor of 32 x 1024 beams through 380k Gaussians 0.53 ms
+// against 7.4 (there the slowest packet was the time), 16 sensors through 580k 6.0 ms against 28.
+__global__ void __launch_bounds__(kRayWarps * 32) k_lidar_trace(const LidarTreeDev* __restrict__ trees,
+                                                                const LidarSlot* __restrict__ slots, int K,
+                                                                const float* __restrict__ dirs, int n_dirs,
+                                                                int64_t n_rays, LidarParams LP,
+                                                                float* __restrict__ out_d, float* __restrict__ out_a,
+                                                                uint32_t* __restrict__ err,
+                                                                unsigned long long* __restrict__ next_ray) {
+    __shared__ RayWarp s_warp[kRayWarps];
+    const int lane = threadIdx.x & 31;
+    RayWarp& W = s_warp[threadIdx.x >> 5];
+    for (;;) {
+        unsigned long long ray = 0;
+        if (lane == 0) ray = atomicAdd(next_ray, 1ull);
+        ray = __shfl_sync(0xffffffffu, ray, 0);
+        if (ray >= (unsigned long long)n_rays) break;
+        const int64_t s = (int64_t)ray / n_dirs, j = (int64_t)ray - s * n_dirs;
+        float ds[3] = {dirs[3 * j], dirs[3 * j + 1], dirs[3 * j + 2]};
+        {
             const float r = rsqrtf(ds[0] * ds[0] + ds[1] * ds[1] + ds[2] * ds[2]);
             ds[0] *= r; ds[1] *= r; ds[2] *= r;
         }
-        const LidarSlot* sl = slots + (int64_t)s * K;
+        const LidarSlot* sl = slots + s * K;
         float T = 1.f, D = 0.f;
-        uint64_t last = 0;                                 // keys <= last are composited
-        bool first = true, done = !valid;
-        while (__any_sync(0xffffffffu, !done)) {
-            int cnt = 0;
-            uint64_t maxkey = ~0ull;                   // key of the last entry once the buffer is full
+        uint64_t last = 0;                             // keys <= last are composited
+        bool first = true, done = false;
+        while (!done) {                                // a round: nearly always the only one
             const float t_lo = first ? LP.r_min : __uint_as_float((uint32_t)(last >> 32));
             float t_hi = LP.r_max;
-            for (int slot = 0; slot < K; ++slot) {
-                int my_node = -1;
-                float o[3] = {0.f, 0.f, 0.f}, d[3] = {1.f, 1.f, 1.f}, id[3] = {1.f, 1.f, 1.f};
-                if (!done) {
-                    const LidarSlot& S = sl[slot];
-                    my_node = S.node;
-                    if (my_node >= 0 && trees[my_node].n == 0) my_node = -1;
-                    if (my_node >= 0) {
-                        for (int a = 0; a < 3; ++a) {
-                            o[a] = S.o[a];
-                            d[a] = S.R[3 * a] * ds[0] + S.R[3 * a + 1] * ds[1] + S.R[3 * a + 2] * ds[2];
-                            id[a] = 1.f / d[a];
-                        }
-                    }
-                }
-                unsigned pending = __ballot_sync(0xffffffffu, my_node >= 0);
-                while (pending) {
-                    const int node = __shfl_sync(0xffffffffu, my_node, __ffs(pending) - 1);
-                    const unsigned mine_mask = __ballot_sync(0xffffffffu, my_node == node) & pending;
-                    pending &= ~mine_mask;
-                    const bool mine = (mine_mask >> lane) & 1u;
-                    const LidarTreeDev tr = trees[node];
-                    int sp = 0;
-                    if (__any_sync(0xffffffffu, mine && slab(tr.box[2], tr.box[3], o, id, t_lo, t_hi))) {
-                        if (lane == 0) stk[0] = 1;
-                        sp = 1;
-                    }
-                    __syncwarp();
-                    while (sp > 0) {
-                        const int64_t k = stk[--sp];
-                        __syncwarp();                        // every lane has read before lane 0 writes
-                        if (k >= tr.P) {
-                            const int64_t g0 = (k - tr.P) * kLeaf;
-                            const int64_t g1 = min(g0 + kLeaf, tr.n);
-                            // the next Gaussian's record is loaded while this one is tested
-                            float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0, n2 = n0, n3 = n0;
-                            if (g0 < g1) {
-                                n0 = __ldg(tr.rec + 4 * g0); n1 = __ldg(tr.rec + 4 * g0 + 1);
-                                n2 = __ldg(tr.rec + 4 * g0 + 2); n3 = __ldg(tr.rec + 4 * g0 + 3);
-                            }
-                            for (int64_t g = g0; g < g1; ++g) {
-                                const float4 r0 = n0, r1 = n1, r2 = n2, r3 = n3;
-                                if (g + 1 < g1) {
-                                    n0 = __ldg(tr.rec + 4 * (g + 1)); n1 = __ldg(tr.rec + 4 * (g + 1) + 1);
-                                    n2 = __ldg(tr.rec + 4 * (g + 1) + 2); n3 = __ldg(tr.rec + 4 * (g + 1) + 3);
-                                }
-                                if (!mine) continue;
-                                const float v0 = o[0] - r0.x, v1 = o[1] - r0.y, v2 = o[2] - r0.z;
-                                {
-                                    const float x0 = fmaf(v1, d[2], -v2 * d[1]), x1 = fmaf(v2, d[0], -v0 * d[2]),
-                                                x2 = fmaf(v0, d[1], -v1 * d[0]);
-                                    if (fmaf(x0, x0, fmaf(x1, x1, x2 * x2)) > r3.y) continue;   // |d| = 1 up to rounding
-                                }
-                                const float op0 = fmaf(r1.x, v0, fmaf(r1.y, v1, r1.z * v2));
-                                const float op1 = fmaf(r1.w, v0, fmaf(r2.x, v1, r2.y * v2));
-                                const float op2 = fmaf(r2.z, v0, fmaf(r2.w, v1, r3.x * v2));
-                                const float dp0 = fmaf(r1.x, d[0], fmaf(r1.y, d[1], r1.z * d[2]));
-                                const float dp1 = fmaf(r1.w, d[0], fmaf(r2.x, d[1], r2.y * d[2]));
-                                const float dp2 = fmaf(r2.z, d[0], fmaf(r2.w, d[1], r3.x * d[2]));
-                                const float dd = fmaf(dp0, dp0, fmaf(dp1, dp1, dp2 * dp2));
-                                const float od = fmaf(op0, dp0, fmaf(op1, dp1, op2 * dp2));
-                                const float c0 = fmaf(op1, dp2, -op2 * dp1), c1 = fmaf(op2, dp0, -op0 * dp2),
-                                            c2 = fmaf(op0, dp1, -op1 * dp0);
-                                const float idd = 1.f / dd;
-                                const float t = -od * idd;
-                                const float q = fmaf(c0, c0, fmaf(c1, c1, c2 * c2)) * idd;
-                                if (!(q <= LP.q_max) || !(t >= LP.r_min) || !(t <= LP.r_max)) continue;
-                                const uint64_t key = ((uint64_t)__float_as_uint(t) << 32) | (uint32_t)(tr.gbase + g);
-                                if ((!first && key <= last) || key >= maxkey) continue;
-                                const float alpha = fminf(LP.alpha_max, r0.w * fast_exp2(kHalfLog2e * q));
-                                if (alpha < LP.alpha_min) continue;
-                                // insert in order; a full buffer drops its last entry
-                                int i = cnt < kKbuf ? cnt : kKbuf - 1;
-                                while (i > 0) {
-                                    const uint32_t pt = kt[(i - 1) * kTraceThreads], pg = kg[(i - 1) * kTraceThreads];
-                                    if ((((uint64_t)pt << 32) | pg) < key) break;
-                                    kt[i * kTraceThreads] = pt;
-                                    kg[i * kTraceThreads] = pg;
-                                    ka[i * kTraceThreads] = ka[(i - 1) * kTraceThreads];
-                                    --i;
-                                }
-                                kt[i * kTraceThreads] = (uint32_t)(key >> 32);
-                                kg[i * kTraceThreads] = (uint32_t)key;
-                                ka[i * kTraceThreads] = alpha;
-                                if (cnt < kKbuf) ++cnt;
-                                if (cnt == kKbuf) {
-                                    const uint32_t lt = kt[(kKbuf - 1) * kTraceThreads];
-                                    maxkey = ((uint64_t)lt << 32) | kg[(kKbuf - 1) * kTraceThreads];
-                                    t_hi = __uint_as_float(lt);
-                                }
-                            }
-                        } else {
-                            const int64_t c = 2 * k;
-                            const float4 l0 = __ldg(tr.box + 2 * c), h0 = __ldg(tr.box + 2 * c + 1),
-                                         l1 = __ldg(tr.box + 2 * c + 2), h1 = __ldg(tr.box + 2 * c + 3);
-                            const bool in0 = mine && slab(l0, h0, o, id, t_lo, t_hi);
-                            const bool in1 = mine && slab(l1, h1, o, id, t_lo, t_hi);
-                            const unsigned b0 = __ballot_sync(0xffffffffu, in0), b1 = __ballot_sync(0xffffffffu, in1);
-                            if (b0 && b1) {
-                                const bool near0 = slab_enter(l0, h0, o, id) <= slab_enter(l1, h1, o, id);
-                                const bool n0 = __shfl_sync(0xffffffffu, near0, __ffs(b0 | b1) - 1);
-                                if (sp + 2 > kStack) {
-                                    if (lane == 0) atomicOr(err, kErrCapacity);
-                                    break;
-                                }
-                                if (lane == 0) {
-                                    stk[sp] = (int)(n0 ? c + 1 : c);     // far child below, near on top
-                                    stk[sp + 1] = (int)(n0 ? c : c + 1);
-                                }
-                                sp += 2;
-                            } else if (b0 || b1) {
-                                if (sp + 1 > kStack) {
-                                    if (lane == 0) atomicOr(err, kErrCapacity);
-                                    break;
-                                }
-                                if (lane == 0) stk[sp] = (int)(b0 ? c : c + 1);
-                                sp += 1;
-                            }
-                            __syncwarp();
+            uint64_t maxkey = ~0ull;                   // farthest kept key once the buffer was cut
+            int cnt = 0, sp = 0, next_slot = 0, flush_at = 32, cur = -1;
+            NodeRay R{};
+            LidarTreeDev tr{};
+            int levels = 0;
+            while (!done) {
+                if (sp == 0) {
+                    if (next_slot >= K) break;
+                    // the roots of the next 32 slots, one per lane
+                    const int slot = next_slot + lane;
+                    bool in = false;
+                    float en = 0.f;
+                    if (slot < K) {
+                        const LidarSlot& S = sl[slot];
+                        if (S.node >= 0 && trees[S.node].n > 0) {
+                            const NodeRay r = node_ray(S, ds);
+                            const float4 lo = trees[S.node].box[2], hi = trees[S.node].box[3];
+                            in = slab(lo, hi, r.o, r.id, t_lo, t_hi);
+                            en = fmaxf(slab_enter(lo, hi, r.o, r.id), t_lo) + 0.f;   // (never -0: ordered as bits below)
                         }
                     }
                     __syncwarp();
+                    push_sorted(W, sp, in, en, 1u, (uint32_t)slot, lane);
+                    next_slot += 32;
+                    continue;
                 }
-            }
-            if (!done) {
-                // composite this round's hits in order
-                for (int i = 0; i < cnt && !done; ++i) {
-                    const float a = ka[i * kTraceThreads];
-                    const float Tn = fmaf(-a, T, T);
-                    if (Tn < LP.t_min) {
+                const uint32_t node = W.node[sp - 1], slot = W.slot[sp - 1];
+                const float enter = W.enter[sp - 1];
+                if (enter > t_hi) { --sp; continue; }
+                if ((int)slot != cur) {
+                    cur = (int)slot;
+                    const LidarSlot& S = sl[cur];
+                    R = node_ray(S, ds);
+                    tr = trees[S.node];
+                    levels = 63 - __clzll(tr.P);
+                }
+                if ((int64_t)node < tr.P) {
+                    const int below = levels - (31 - __clz(node));          // levels left to the leaves, >= 1
+                    const int st = below % 5 ? below % 5 : 5;
+                    const uint32_t child = (node << st) + (uint32_t)lane;
+                    --sp;
+                    bool in = false;
+                    float en = 0.f;
+                    if (lane < (1 << st)) {
+                        const float4 lo = __ldg(tr.box + 2 * (size_t)child), hi = __ldg(tr.box + 2 * (size_t)child + 1);
+                        in = slab(lo, hi, R.o, R.id, t_lo, t_hi);
+                        en = fmaxf(slab_enter(lo, hi, R.o, R.id), t_lo) + 0.f;
+                    }
+                    __syncwarp();                      // every lane has read the popped entry
+                    if (sp + 32 > kStack) {            // cannot happen for trees of the documented sizes
+                        if (lane == 0) atomicOr(err, kErrCapacity);
                         done = true;
-                    } else {
-                        D = fmaf(a * T, __uint_as_float(kt[i * kTraceThreads]), D);
-                        T = Tn;
+                        break;
+                    }
+                    push_sorted(W, sp, in, en, child, slot, lane);
+                    continue;
+                }
+                // the leaves of this slot on top of the stack, at most four
+                const int at = sp - 1 - lane;
+                const unsigned lm = __ballot_sync(0xffffffffu, lane < 4 && at >= 0 && W.slot[max(at, 0)] == slot &&
+                                                                   (int64_t)W.node[max(at, 0)] >= tr.P);
+                const int nl = __ffs(~lm) - 1, li = lane >> 3;
+                int64_t g = -1;
+                if (li < nl && W.enter[sp - 1 - li] <= t_hi)
+                    g = ((int64_t)W.node[sp - 1 - li] - tr.P) * kLeaf + (lane & (kLeaf - 1));
+                sp -= nl;
+                __syncwarp();
+                bool hit = false;
+                float t = 0.f, alpha = 0.f;
+                if (g >= 0 && g < tr.n) {
+                    const float4* rp = tr.rec + 4 * g;
+                    const float4 r0 = __ldg(rp), r1 = __ldg(rp + 1), r2 = __ldg(rp + 2), r3 = __ldg(rp + 3);
+                    const float v0 = R.o[0] - r0.x, v1 = R.o[1] - r0.y, v2 = R.o[2] - r0.z;
+                    const float x0 = fmaf(v1, R.d[2], -v2 * R.d[1]), x1 = fmaf(v2, R.d[0], -v0 * R.d[2]),
+                                x2 = fmaf(v0, R.d[1], -v1 * R.d[0]);
+                    if (!(fmaf(x0, x0, fmaf(x1, x1, x2 * x2)) > r3.y)) {   // |d| = 1 up to rounding
+                        const float op0 = fmaf(r1.x, v0, fmaf(r1.y, v1, r1.z * v2));
+                        const float op1 = fmaf(r1.w, v0, fmaf(r2.x, v1, r2.y * v2));
+                        const float op2 = fmaf(r2.z, v0, fmaf(r2.w, v1, r3.x * v2));
+                        const float dp0 = fmaf(r1.x, R.d[0], fmaf(r1.y, R.d[1], r1.z * R.d[2]));
+                        const float dp1 = fmaf(r1.w, R.d[0], fmaf(r2.x, R.d[1], r2.y * R.d[2]));
+                        const float dp2 = fmaf(r2.z, R.d[0], fmaf(r2.w, R.d[1], r3.x * R.d[2]));
+                        const float dd = fmaf(dp0, dp0, fmaf(dp1, dp1, dp2 * dp2));
+                        const float od = fmaf(op0, dp0, fmaf(op1, dp1, op2 * dp2));
+                        const float c0 = fmaf(op1, dp2, -op2 * dp1), c1 = fmaf(op2, dp0, -op0 * dp2),
+                                    c2 = fmaf(op0, dp1, -op1 * dp0);
+                        const float idd = 1.f / dd;
+                        t = -od * idd;
+                        const float q = fmaf(c0, c0, fmaf(c1, c1, c2 * c2)) * idd;
+                        if (q <= LP.q_max && t >= LP.r_min && t <= LP.r_max) {
+                            const uint64_t key = ((uint64_t)__float_as_uint(t) << 32) | (uint32_t)(tr.gbase + g);
+                            if ((first || key > last) && key < maxkey) {
+                                alpha = fminf(LP.alpha_max, r0.w * fast_exp2(kHalfLog2e * q));
+                                hit = alpha >= LP.alpha_min;
+                            }
+                        }
                     }
                 }
-                if (cnt < kKbuf) done = true;
-                last = maxkey;
-                first = false;
+                const unsigned hm = __ballot_sync(0xffffffffu, hit);
+                if (hm == 0) continue;
+                if (hit) {
+                    const int p = cnt + __popc(hm & ((1u << lane) - 1u));
+                    W.t[p] = __float_as_uint(t);
+                    W.g[p] = (uint32_t)(tr.gbase + g);
+                    W.a[p] = alpha;
+                }
+                cnt += __popc(hm);
+                __syncwarp();
+                if (cnt < flush_at) continue;
+                // final hits: before the entry of every node left, less a margin for the rounding of
+                // the boxes' entries and of t* (hits of unvisited slots may lie anywhere)
+                if (next_slot >= K) {
+                    float bound = INFINITY;
+                    for (int i = lane; i < sp; i += 32) bound = fminf(bound, W.enter[i]);
+                    bound = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(bound)));   // >= 0: ordered as bits
+                    done = composite_pending(W, cnt, fmaf(bound, 1.f - 1e-5f, -1e-5f), LP.t_min, lane, T, D);
+                    if (done) break;
+                }
+                if (cnt > kPend - 32) {
+                    maxkey = cut_pending(W, cnt, lane);
+                    t_hi = __uint_as_float((uint32_t)(maxkey >> 32));
+                }
+                flush_at = min(cnt + 24, kPend - 31);
             }
+            if (done) break;
+            if (composite_pending(W, cnt, INFINITY, LP.t_min, lane, T, D) || maxkey == ~0ull) break;
+            last = maxkey;
+            first = false;
         }
-        if (valid) {
+        if (lane == 0) {
             out_d[ray] = D;
             out_a[ray] = 1.f - T;
         }
+        __syncwarp();
     }
 }
 
@@ -425,22 +531,16 @@ void launch_lidar_trace(const Launch& L, const LidarTreeDev* trees, const LidarS
     if (n_rays <= 0) return;
     static int resident = 0, sms = 0;           // blocks per SM at this kernel's resources
     if (!resident) {
-        int dev = 0;
+        int dev = 0, r = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaFuncSetAttribute(k_lidar_trace, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kKbufBytes);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k_lidar_trace, kTraceThreads, kKbufBytes);
-        resident = std::max(resident, 1);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, k_lidar_trace, kRayWarps * 32, 0);
+        resident = std::max(r, 1);
     }
-    const int64_t need = (n_rays + kTraceThreads - 1) / kTraceThreads;
+    const int64_t need = (n_rays + kRayWarps - 1) / kRayWarps;
     const unsigned blocks = (unsigned)std::min<int64_t>(need, (int64_t)resident * sms);
-    const unsigned long long n_packets = (unsigned long long)(n_rays + 31) / 32;
-    unsigned long long a = 0x9E3779B97F4A7C15ull % n_packets;          // a multiplier coprime with n_packets
-    auto gcd = [](unsigned long long x, unsigned long long y) { while (y) { const auto t = x % y; x = y; y = t; } return x; };
-    if (a == 0) a = 1;
-    while (gcd(a, n_packets) != 1) ++a;
-    k_lidar_trace<<<blocks, kTraceThreads, kKbufBytes, L.stream>>>(trees, slots, K, dirs, n_dirs, n_rays, LP, out_d,
-                                                                   out_a, err, next_ray, n_packets, a);
+    k_lidar_trace<<<blocks, kRayWarps * 32, 0, L.stream>>>(trees, slots, K, dirs, n_dirs, n_rays, LP, out_d, out_a, err,
+                                                           next_ray);
     ++*L.launches;
 }
 
