@@ -2089,31 +2089,35 @@ int dgs_tsdf_integrate(dgs_ctx* ctx, float* tsdf, float* weight, int32_t nx, int
             for (int b = 0; b < 3; ++b) tv.R[3 * a + b] = c.cam_from_world[4 * a + b];
             tv.t[a] = c.cam_from_world[4 * a + 3];
         }
-        tv.fx = c.fx; tv.fy = c.fy; tv.cx = c.cx; tv.cy = c.cy; tv.W = c.width; tv.H = c.height;
+        tv.fx = c.fx; tv.fy = c.fy; tv.cx = c.cx + 0.f; tv.cy = c.cy + 0.f;   // (-0 becomes +0: see in_range)
+        tv.W = c.width; tv.H = c.height; tv.Wf = (float)c.width; tv.Hf = (float)c.height;
         tv.pix_off = view_pixel_offset ? view_pixel_offset[v] : packed;
         if (tv.pix_off < 0) return fail(ctx, DGS_ERR_INVALID_ARG, "negative view_pixel_offset");
         tv.q0 = packed;
         packed += (int64_t)c.width * c.height;
     }
     cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
-    const size_t bytes = sizeof(TsdfView) * n_views;
+    const size_t bytes = n_views > kTsdfParamViews ? sizeof(TsdfView) * n_views : 0;   // fewer travel with the launch
     const uint64_t gen = ctx->gen;               // read by this call only, never by a captured graph
-    int rc = ensure(ctx, ctx->tsdf_meta, bytes);
+    int rc = bytes ? ensure(ctx, ctx->tsdf_meta, bytes) : DGS_OK;
     if (!rc) rc = ensure(ctx, ctx->tsdf_depth, sizeof(float) * packed);
     ctx->gen = gen;
     if (rc) return rc;
-    if ((rc = ensure_host(ctx, ctx->h_tsdf, ctx->h_tsdf_bytes, bytes))) return rc;
-    if (!ctx->tsdf_copied) DGS_CUDA(ctx, cudaEventCreateWithFlags(&ctx->tsdf_copied, cudaEventDisableTiming));
-    else DGS_CUDA(ctx, cudaEventSynchronize(ctx->tsdf_copied));
-    std::memcpy(ctx->h_tsdf, views.data(), bytes);
-    DGS_CUDA(ctx, cudaMemcpyAsync(ctx->tsdf_meta.p, ctx->h_tsdf, bytes, cudaMemcpyHostToDevice, stream));
-    DGS_CUDA(ctx, cudaEventRecord(ctx->tsdf_copied, stream));
+    if (bytes) {
+        if ((rc = ensure_host(ctx, ctx->h_tsdf, ctx->h_tsdf_bytes, bytes))) return rc;
+        if (!ctx->tsdf_copied) DGS_CUDA(ctx, cudaEventCreateWithFlags(&ctx->tsdf_copied, cudaEventDisableTiming));
+        else DGS_CUDA(ctx, cudaEventSynchronize(ctx->tsdf_copied));
+        std::memcpy(ctx->h_tsdf, views.data(), bytes);
+        DGS_CUDA(ctx, cudaMemcpyAsync(ctx->tsdf_meta.p, ctx->h_tsdf, bytes, cudaMemcpyHostToDevice, stream));
+        DGS_CUDA(ctx, cudaEventRecord(ctx->tsdf_copied, stream));
+    }
     TsdfParams TP{origin[0], origin[1], origin[2], voxel, trunc, 1.f / trunc, max_weight, min_alpha};
     Launch L{stream, &ctx->launches};
     Timer tm{ctx, stream, ctx->opt.profile != 0};
     tm.begin(DGS_K_TSDF);
-    launch_tsdf(L, tsdf, weight, nx, ny, (int64_t)nx * ny * nz, TP, static_cast<const TsdfView*>(ctx->tsdf_meta.p),
-                n_views, depth, alpha, static_cast<float*>(ctx->tsdf_depth.p), packed);
+    launch_tsdf(L, tsdf, weight, nx, ny, (int64_t)nx * ny * nz, TP, views.data(),
+                static_cast<const TsdfView*>(ctx->tsdf_meta.p), n_views, depth, alpha,
+                static_cast<float*>(ctx->tsdf_depth.p));
     tm.end();
     DGS_CUDA(ctx, cudaGetLastError());
     if (ctx->opt.profile) {

@@ -596,14 +596,22 @@ struct TsdfView {
     float R[9], t[3];        // cam_from_world
     float fx, fy, cx, cy;
     int32_t W, H;
+    float Wf, Hf;            // W and H as floats
     int64_t pix_off;         // first pixel of the view in the depth / coverage arrays
     int64_t q0;              // first pixel of the view in the packed normalised-depth scratch
 };
 struct TsdfParams {
     float ox, oy, oz, voxel, trunc, inv_trunc, max_weight, min_alpha;
 };
+// host_views: the V views; up to kTsdfParamViews of them travel as a kernel parameter, more are
+// read from table (the same views in device memory).  dn: scratch of one float per pixel.
+constexpr int kTsdfParamViews = 40;
+struct TsdfViews {
+    TsdfView v[kTsdfParamViews];
+};
 void launch_tsdf(const Launch& L, float* F, float* W, int nx, int ny, int64_t n_vox, const TsdfParams& TP,
-                 const TsdfView* views, int V, const float* depth, const float* alpha, float* dn, int64_t n_pix);
+                 const TsdfView* host_views, const TsdfView* table, int V, const float* depth, const float* alpha,
+                 float* dn);
 
 void launch_composite_bwd(const Launch& L, const ViewDesc* views, int v0, int n_group_views, int n_tiles,
                           const uint2* ranges, const uint32_t* keys, const uint32_t* vals, const Record* records,
