@@ -1647,7 +1647,7 @@ int enqueue_adjoint(dgs_ctx* ctx, const Batch& B, const GroupLists& G, const flo
                     cudaStream_t stream, Timer& tm) {
     Launch L{stream, &ctx->launches};
     tm.begin(DGS_K_BACKWARD);
-    DGS_CUDA(ctx, cudaMemsetAsync(ctx->inst_grad.p, 0, sizeof(float) * 10 * std::max<uint32_t>(G.n_inst, 1), stream));
+    DGS_CUDA(ctx, cudaMemsetAsync(ctx->inst_grad.p, 0, sizeof(float) * kInstGrad * std::max<uint32_t>(G.n_inst, 1), stream));
     launch_composite_bwd(L, B.d_views, G.v0, G.v1 - G.v0, G.n_tiles, static_cast<uint2*>(G.lb->ranges.p), G.keys, G.vals,
                          static_cast<Record*>(G.lb->records.p), G.P, out_rgb, out_depth, grad_rgb, grad_depth,
                          static_cast<float*>(ctx->inst_grad.p), n_red, G.order, G.ck, G.n_jobs_bound);
@@ -1708,7 +1708,7 @@ int dgs_render_backward(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nodes, co
         for (const GroupLists& G : S->groups) max_inst = std::max<uint64_t>(max_inst, G.n_inst);
     else
         for (auto& g : B.groups) max_inst = std::max<uint64_t>(max_inst, B.inst_at[g.second] - B.inst_at[g.first]);
-    if ((rc = ensure(ctx, ctx->inst_grad, sizeof(float) * 10 * max_inst))) return rc;
+    if ((rc = ensure(ctx, ctx->inst_grad, sizeof(float) * kInstGrad * max_inst))) return rc;
     if (ctx->opt.profile >= 2) {
         n_red = reinterpret_cast<unsigned long long*>(static_cast<char*>(ctx->errword.p) + 56);
         DGS_CUDA(ctx, cudaMemsetAsync(n_red, 0, sizeof(unsigned long long), stream));

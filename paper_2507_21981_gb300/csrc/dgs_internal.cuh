@@ -259,6 +259,27 @@ __device__ __forceinline__ float fast_log2(float x) {
     return y;
 }
 
+// Packed FP32 pairs (one issue slot for two lanes' worth of arithmetic, each half rounded as the
+// scalar instruction rounds it).
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    float2 d;
+    asm("{.reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n add.rn.f32x2 z, x, y;\n mov.b64 {%0, %1}, z;}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    float2 d;
+    asm("{.reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n mul.rn.f32x2 z, x, y;\n mov.b64 {%0, %1}, z;}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("{.reg .b64 x, y, z, w;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n mov.b64 w, {%6, %7};\n fma.rn.f32x2 z, x, y, w;\n mov.b64 {%0, %1}, z;}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+
 // Sec. III-A cutoffs of a record at a pixel, as one threshold on the exponent p (alpha =
 // min(alpha_max, o 2^p)): the pixel is skipped unless p >= max(p_min, log2(alpha_min) - log2 o),
 // i.e. unless it lies inside the 3-sigma ellipse and its alpha reaches alpha_min.  Taken in the
@@ -612,6 +633,9 @@ struct TsdfViews {
 void launch_tsdf(const Launch& L, float* F, float* W, int nx, int ny, int64_t n_vox, const TsdfParams& TP,
                  const TsdfView* host_views, const TsdfView* table, int V, const float* depth, const float* alpha,
                  float* dn);
+
+// Floats per instance of the adjoint's accumulators: the ten partials in three 16-byte quads.
+constexpr int kInstGrad = 12;
 
 void launch_composite_bwd(const Launch& L, const ViewDesc* views, int v0, int n_group_views, int n_tiles,
                           const uint2* ranges, const uint32_t* keys, const uint32_t* vals, const Record* records,
