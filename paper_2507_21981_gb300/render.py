@@ -235,7 +235,9 @@ class Renderer:
         if self.mode != "graph":
             return fresh()
         o = self._outs
-        if o is None or o[1].numel() != ds.n_pixels or o[1].device != ds.device or (o[2] is not None) != with_alpha:
+        # (the tensors' device: ds.device may name no index, "cuda", and then equals no tensor's)
+        if o is None or o[1].numel() != ds.n_pixels or o[1].device != ds.node_poses.device or \
+                (o[2] is not None) != with_alpha:
             self._outs = o = fresh()
         return o
 
