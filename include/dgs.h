@@ -222,7 +222,7 @@ int dgs_workspace_query(const dgs_ctx* ctx, size_t* bytes);
  * kernels on `stream` (allocating the tables they need in the context, as a render would),
  * reads the totals back and writes to *bytes the sum of the count tables and of the tile lists of
  * its view groups (two list sets when the batch runs as two or more groups), without allocating
- * the lists.  The adjoint needs 40 bytes per visible instance of its largest view group on top.
+ * the lists.  The adjoint needs 48 bytes per visible instance of its largest view group on top.
  * Synchronises `stream`.
  */
 int dgs_workspace_query_batch(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nodes, const int32_t* env_node_ids,

@@ -50,15 +50,15 @@ struct GraphKey {
 };
 
 // Workspace of one view group's lists.  dkey/ival: depth keys and instance numbers (depth
-// sort, ping-pong); ntile: pairs per instance; poff/tparts: pair offsets in depth order;
-// tkeys/tvals: (tile, instance) pairs (tile sort, ping-pong); ranges: per tile.
+// sort, ping-pong); ntile: pairs per instance; poff: pair offsets in depth order; tkeys/tvals:
+// (tile, instance) pairs (tile sort, ping-pong); scratch: the words that start at zero (ListPlan),
+// the ranges per tile among them.
 struct ListBufs {
-    DevBuf records, info, dkey0, ival0, dkey1, ival1, ntile, poff, tparts, tkeys0, tvals0, tkeys1, tvals1, hist,
-        status, counters, ranges, torder, ck_st, ck_off, ck_last, ck_jobs, ck_njobs, vig;
-    static constexpr int kCount = 24;
-    DevBuf* all[kCount] = {&records, &info, &dkey0, &ival0, &dkey1, &ival1, &ntile, &poff, &tparts, &tkeys0, &tvals0,
-                           &tkeys1, &tvals1, &hist, &status, &counters, &ranges, &torder, &ck_st, &ck_off, &ck_last,
-                           &ck_jobs, &ck_njobs, &vig};
+    DevBuf records, info, dkey0, ival0, dkey1, ival1, ntile, poff, tkeys0, tvals0, tkeys1, tvals1, scratch, torder,
+        ck_st, ck_off, ck_last, ck_jobs, ck_njobs, vig;
+    static constexpr int kCount = 20;
+    DevBuf* all[kCount] = {&records, &info, &dkey0, &ival0, &dkey1, &ival1, &ntile, &poff, &tkeys0, &tvals0,
+                           &tkeys1, &tvals1, &scratch, &torder, &ck_st, &ck_off, &ck_last, &ck_jobs, &ck_njobs, &vig};
     ListBufs() = default;
     ListBufs(const ListBufs&) = delete;
     ListBufs& operator=(const ListBufs&) = delete;
@@ -73,7 +73,7 @@ struct dgs_ctx {
     std::unique_ptr<SavedForward> saved;  // valid until the next call stages a batch
     std::string err;
     int device = 0;
-    DevBuf meta, counts, inst_off, pair_off, parts, errword, readback, inst_grad, gsizes, totals;
+    DevBuf meta, counts, inst_off, pair_off, parts, errword, readback, inst_grad;
     ListBufs lists[2];                    // view groups alternate between two sets (two streams)
     cudaStream_t aux_stream = nullptr;    // second stream of the eager sequence
     uint64_t gen = 0;                     // bumped whenever a workspace buffer is reallocated
@@ -91,6 +91,7 @@ struct dgs_ctx {
     const uint32_t* gkeys[2] = {nullptr, nullptr};
     const uint32_t* gvals[2] = {nullptr, nullptr};
     const uint32_t* gorder[2] = {nullptr, nullptr};
+    const uint2* granges[2] = {nullptr, nullptr};
     Params gP[2]{};
     Checkpoints gck[2]{};
     uint32_t gjobs[2] = {0, 0};
@@ -98,6 +99,7 @@ struct dgs_ctx {
     void* h_graph = nullptr;              // pinned: error word + live totals after a replay
     void* h_meta = nullptr;
     size_t h_meta_bytes = 0;
+    cudaEvent_t meta_copied = nullptr;    // the staging's last upload has been read
     void* h_read = nullptr;
     size_t h_read_bytes = 0;
     dgs_stats stats{};
@@ -256,13 +258,22 @@ void collect_times(dgs_ctx* ctx) {
 // receives the 64-bit instance total of the count scan (the 32-bit offsets wrap beyond 2^32).
 __global__ void k_view_totals(const uint32_t* __restrict__ inst_off, const uint64_t* __restrict__ pair_off,
                               const int64_t* __restrict__ view_tab, int n, const ulonglong2* __restrict__ scan_total,
-                              uint64_t* out) {
+                              const uint32_t* __restrict__ err, uint64_t* out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     out[i] = inst_off[view_tab[i]];
     out[n + i] = pair_off[view_tab[i]];
-    if (i == 0) out[2 * n + 1] = scan_total ? scan_total->x : 0ull;
+    if (i == 0) {
+        out[2 * n] = *err;
+        out[2 * n + 1] = scan_total ? scan_total->x : 0ull;
+    }
 }
+
+// The error word's buffer: the error block, the graph replay's sizes, then the exact pairs of every
+// view group, so that one copy reads a call's results back.
+constexpr size_t kSizesAt = kErrBlockBytes / 4, kTotalsAt = kSizesAt + 32;   // in words
+uint32_t* sizes_of(uint32_t* err) { return err + kSizesAt; }
+uint32_t* totals_of(uint32_t* err) { return err + kTotalsAt; }
 
 constexpr uint64_t kPipelinePairs = 1ull << 22;   // batches with this many pairs run as two groups
 
@@ -570,8 +581,9 @@ int stage(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nodes, const int32_t* e
     int rc;
     if ((rc = ensure(ctx, ctx->meta, meta_bytes))) return rc;
     if ((rc = ensure_host(ctx, ctx->h_meta, ctx->h_meta_bytes, upload_bytes))) return rc;
-    // the previous call's upload may still be in flight from this staging buffer
-    DGS_CUDA(ctx, cudaStreamSynchronize(stream));
+    // a previous call's upload may still be in flight from this staging buffer
+    if (!ctx->meta_copied) DGS_CUDA(ctx, cudaEventCreateWithFlags(&ctx->meta_copied, cudaEventDisableTiming));
+    else DGS_CUDA(ctx, cudaEventSynchronize(ctx->meta_copied));
     char* hm = static_cast<char*>(ctx->h_meta);
     std::memcpy(hm + o_nodes, nd.data(), sizeof(NodeDesc) * n_nodes);
     std::memcpy(hm + o_views, views.data(), sizeof(ViewDesc) * V);
@@ -595,23 +607,22 @@ int stage(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nodes, const int32_t* e
     const int64_t* d_viewtab = reinterpret_cast<const int64_t*>(dm + o_viewtab);
     VNode* d_vnodes = reinterpret_cast<VNode*>(dm + o_vnodes);
 
-    if ((rc = ensure(ctx, ctx->errword, kErrBlockBytes))) return rc;
+    if ((rc = ensure(ctx, ctx->errword, sizeof(uint32_t) * (kTotalsAt + V + 1)))) return rc;
     if ((rc = ensure(ctx, ctx->counts, sizeof(uint2) * std::max<int64_t>(T, 1)))) return rc;
     if ((rc = ensure(ctx, ctx->inst_off, sizeof(uint32_t) * (T + 1)))) return rc;
     if ((rc = ensure(ctx, ctx->pair_off, sizeof(uint64_t) * (T + 1)))) return rc;
     const int64_t n_parts = (T + 4095) / 4096;
     if ((rc = ensure(ctx, ctx->parts, sizeof(ulonglong2) * (n_parts + 1)))) return rc;
     if ((rc = ensure(ctx, ctx->readback, sizeof(uint64_t) * 2 * (V + 1) + 64))) return rc;
-    // pinned: per-view totals, the error word, then the exact pairs of every view group (<= V)
-    if ((rc = ensure_host(ctx, ctx->h_read, ctx->h_read_bytes, sizeof(uint64_t) * 2 * (V + 1) + 64 + 4 * (V + 1))))
+    // pinned: per-view totals, then the error word's buffer
+    if ((rc = ensure_host(ctx, ctx->h_read, ctx->h_read_bytes, sizeof(uint64_t) * 2 * (V + 1) + 4 * (kTotalsAt + V + 1))))
         return rc;
-    if ((rc = ensure(ctx, ctx->totals, sizeof(uint32_t) * (V + 1)))) return rc;
-    B.front_bytes = meta_bytes + 64 + sizeof(uint2) * std::max<int64_t>(T, 1) + sizeof(uint32_t) * (T + 1) +
-                    sizeof(uint64_t) * (T + 1) + sizeof(ulonglong2) * (n_parts + 1) + sizeof(uint64_t) * 2 * (V + 1) +
-                    64 + sizeof(uint32_t) * (V + 1);
+    B.front_bytes = meta_bytes + sizeof(uint32_t) * (kTotalsAt + V + 1) + sizeof(uint2) * std::max<int64_t>(T, 1) + sizeof(uint32_t) * (T + 1) +
+                    sizeof(uint64_t) * (T + 1) + sizeof(ulonglong2) * (n_parts + 1) + sizeof(uint64_t) * 2 * (V + 1) + 64;
     uint32_t* d_err = static_cast<uint32_t*>(ctx->errword.p);
 
     DGS_CUDA(ctx, cudaMemcpyAsync(dm, hm, upload_bytes, cudaMemcpyHostToDevice, stream));
+    DGS_CUDA(ctx, cudaEventRecord(ctx->meta_copied, stream));
 
     Params P = make_params(o);
     P.err = d_err;
@@ -692,10 +703,10 @@ void list_bytes(uint64_t n_inst, uint64_t n_pairs, int64_t n_tiles, int tile_px,
     const size_t n_sub = (size_t)tile_px / 32;
     const size_t b[ListBufs::kCount] = {
         sizeof(Record) * n_inst, sizeof(InstInfo) * n_inst, u * n_inst, u * n_inst, u * n_inst,
-        u * n_inst, u * n_inst, u * (n_inst + 1), u * tile_scan_parts((uint32_t)n_inst),
-        u * n_pairs, u * n_pairs, u * n_pairs, u * n_pairs, u * 4 * 1024,
-        u * sort_status_words((uint32_t)std::max(n_inst, n_pairs)), u * 8,
-        sizeof(uint2) * nt, n_tiles <= kOrderMaxTiles ? u * nt : 0,
+        u * n_inst, u * n_inst, u * (n_inst + 1),
+        u * n_pairs, u * n_pairs, u * n_pairs, u * n_pairs,
+        u * list_scratch_bound((uint32_t)n_inst, (uint32_t)n_pairs, n_tiles),
+        n_tiles <= kOrderMaxTiles ? u * nt : 0,
         ck, ck ? u * nt : 0, ck ? u * nt * n_sub : 0, ck ? sizeof(uint2) * (nt + ck_slots(n_pairs)) : 0, ck ? u : 0,
         u * n_inst};
     for (int i = 0; i < ListBufs::kCount; ++i) out[i] = b[i];
@@ -723,10 +734,8 @@ int readback_groups(dgs_ctx* ctx, Batch& B, cudaStream_t stream, Timer& tm, size
         uint64_t* d_rb = static_cast<uint64_t*>(ctx->readback.p);
         const ulonglong2* scan_total = B.n_parts > 0 ? static_cast<ulonglong2*>(ctx->parts.p) + B.n_parts : nullptr;
         k_view_totals<<<(V + 1 + 127) / 128, 128, 0, stream>>>(B.d_inst_off, B.d_pair_off, B.d_viewtab, V + 1,
-                                                               scan_total, d_rb);
+                                                               scan_total, B.d_err, d_rb);
         ++ctx->launches;
-        DGS_CUDA(ctx, cudaMemsetAsync(d_rb + 2 * (V + 1), 0, sizeof(uint64_t), stream));
-        DGS_CUDA(ctx, cudaMemcpyAsync(d_rb + 2 * (V + 1), B.d_err, sizeof(uint32_t), cudaMemcpyDeviceToDevice, stream));
         DGS_CUDA(ctx, cudaMemcpyAsync(ctx->h_read, d_rb, sizeof(uint64_t) * 2 * (V + 1) + 16, cudaMemcpyDeviceToHost, stream));
     }
     tm.end();
@@ -828,16 +837,19 @@ int prepare(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nodes, const int32_t*
 // write and the adjoint's (tile, segment) jobs (bounded by *n_jobs_bound); else ck->st is null.
 void enqueue_lists(dgs_ctx* ctx, ListBufs& lb, const Batch& B, const Launch& L, Timer& tm, int v0, int v1, int n_tiles,
                    uint32_t inst_base, uint32_t n_inst, uint32_t n_bound, const uint32_t* d_inst, uint32_t* d_pairs,
-                   const Params& P, const uint32_t** keys, const uint32_t** vals, const uint32_t** tile_order,
-                   Checkpoints* ck, uint32_t* n_jobs_bound, bool want_ck = true) {
+                   const Params& P, const uint32_t** keys, const uint32_t** vals, const uint2** ranges_out,
+                   const uint32_t** tile_order, Checkpoints* ck, uint32_t* n_jobs_bound, bool want_ck = true) {
     const int K = B.K;
     auto u32 = [](DevBuf& b) { return static_cast<uint32_t*>(b.p); };
     Record* rec = static_cast<Record*>(lb.records.p);
     InstInfo* info = static_cast<InstInfo*>(lb.info.p);
-    // the depth sort's view key: packed into the instance numbers where both fit in 32 bits
+    // (test_fault 4: the depth sort gathers the view key, as for groups whose numbers leave no room)
+    const ListPlan plan = plan_lists(n_inst, n_bound, v1 - v0, P.tbits, n_tiles, ctx->opt.test_fault == 4);
+    uint32_t* const scratch = u32(lb.scratch);
+    uint2* const ranges = reinterpret_cast<uint2*>(scratch + plan.ranges);
+    cudaMemsetAsync(scratch, 0, sizeof(uint32_t) * plan.words, L.stream);
     ViewKey vk;
-    vk.bits = bits_for((uint64_t)(v1 - v0));
-    // (test_fault 4: the gathered form, as for groups whose numbers leave no room)
+    vk.bits = plan.view_bits;
     if (vk.bits > 0 && bits_for((uint64_t)n_inst) + vk.bits <= 32 && ctx->opt.test_fault != 4)
         vk.vshift = 32 - vk.bits;
     vk.vig = vk.bits > 0 && !vk.vshift ? u32(lb.vig) : nullptr;
@@ -847,6 +859,7 @@ void enqueue_lists(dgs_ctx* ctx, ListBufs& lb, const Batch& B, const Launch& L, 
     vk.nv = v1 - v0;
     Params Pe = P;
     Pe.vshift = vk.vshift;
+    Pe.vkey = plan.depth_bits > kZBits;
     tm.begin(DGS_K_EMIT);
     launch_emit(L, B.dtype_mask, B.d_nodes, B.n_nodes, B.d_views, B.d_vnodes, K, B.d_nv, B.d_nvoff, (int)B.chunk_total,
                 Pe, v0, v1, B.batched, B.d_pmap + (size_t)v0 * (2 * K + 1), B.view_tab[v0 + 1] - B.view_tab[v0],
@@ -863,21 +876,23 @@ void enqueue_lists(dgs_ctx* ctx, ListBufs& lb, const Batch& B, const Launch& L, 
     depth_ctl.runs = true;  // emission order (view by view, Z-ordered nodes) keeps the high depth digits in runs
     // instances by depth, then by view (most significant, through the values): each view's
     // instances in depth order, so that every instance's pairs come out view by view
-    launch_sort(L, u32(lb.dkey0), u32(lb.ival0), u32(lb.dkey1), u32(lb.ival1), n_inst, kZBits, u32(lb.hist),
-                u32(lb.status), u32(lb.counters), B.d_err, &dk, &order, d_inst, depth_ctl, &vk);
-    launch_tile_scan(L, order, u32(lb.ntile), n_inst, d_inst, u32(lb.poff), u32(lb.tparts), n_bound, d_pairs, B.d_err);
+    launch_sort(L, u32(lb.dkey0), u32(lb.ival0), u32(lb.dkey1), u32(lb.ival1), n_inst, plan.depth_bits,
+                scratch + plan.depth, B.d_err, &dk, &order, d_inst, depth_ctl, &vk);
+    launch_tile_scan(L, order, u32(lb.ntile), n_inst, d_inst, u32(lb.poff), scratch + plan.tscan, n_bound, d_pairs,
+                     B.d_err, ctl.spin_ns);
     launch_pairs(L, B.d_views, K, order, u32(lb.poff), rec, info, n_inst, d_inst, P, u32(lb.tkeys0),
                  u32(lb.tvals0), n_bound);
     uint32_t *tk = nullptr, *tv = nullptr;
     // pairs by tile in view only: stability keeps them view by view within each tile index
-    launch_sort(L, u32(lb.tkeys0), u32(lb.tvals0), u32(lb.tkeys1), u32(lb.tvals1), n_bound, P.tbits, u32(lb.hist),
-                u32(lb.status), u32(lb.counters), B.d_err, &tk, &tv, d_pairs, tile_ctl);
+    launch_sort(L, u32(lb.tkeys0), u32(lb.tvals0), u32(lb.tkeys1), u32(lb.tvals1), n_bound, P.tbits,
+                scratch + plan.tile, B.d_err, &tk, &tv, d_pairs, tile_ctl);
     tm.end();
     tm.begin(DGS_K_RANGES);
-    launch_ranges(L, tk, n_bound, static_cast<uint2*>(lb.ranges.p), n_tiles, d_pairs, B.d_views, v1 - v0, P);
+    launch_ranges(L, tk, n_bound, ranges, n_tiles, d_pairs, B.d_views, v1 - v0, P);
+    *ranges_out = ranges;
     *tile_order = nullptr;
     if (n_tiles <= kOrderMaxTiles && lb.torder.bytes >= sizeof(uint32_t) * (size_t)n_tiles) {
-        launch_tile_order(L, static_cast<uint2*>(lb.ranges.p), n_tiles, static_cast<uint32_t*>(lb.torder.p));
+        launch_tile_order(L, ranges, n_tiles, static_cast<uint32_t*>(lb.torder.p), scratch + plan.order);
         *tile_order = static_cast<uint32_t*>(lb.torder.p);
     }
     *ck = Checkpoints{};
@@ -890,7 +905,7 @@ void enqueue_lists(dgs_ctx* ctx, ListBufs& lb, const Batch& B, const Launch& L, 
         ck->jobs = static_cast<uint2*>(lb.ck_jobs.p);
         ck->n_jobs = u32(lb.ck_njobs);
         *n_jobs_bound = (uint32_t)(n_tiles + ck_slots(n_bound));
-        launch_segment_jobs(L, static_cast<uint2*>(lb.ranges.p), n_tiles, *ck);
+        launch_segment_jobs(L, ranges, n_tiles, *ck);
     }
     tm.end();
     *keys = tk;
@@ -903,6 +918,7 @@ struct GroupLists {
     uint32_t n_bound = 0, n_inst = 0;
     const uint32_t* keys = nullptr;
     const uint32_t* vals = nullptr;
+    const uint2* ranges = nullptr;
     const uint32_t* order = nullptr;      // tiles by descending list length, or null
     Checkpoints ck{};                     // compositor checkpoints (keep_lists), or ck.st null
     uint32_t n_jobs_bound = 0;            // bound on the adjoint's (tile, segment) jobs
@@ -973,7 +989,7 @@ void build_group_lists(dgs_ctx* ctx, const Batch& B, int g, ListBufs& lb, cudaSt
     G.P.n_rec = G.n_inst;
     G.lb = &lb;
     enqueue_lists(ctx, lb, B, L, tm, v0, v1, G.n_tiles, (uint32_t)B.inst_at[v0], G.n_inst, G.n_bound, nullptr,
-                  static_cast<uint32_t*>(ctx->totals.p) + g, G.P, &G.keys, &G.vals, &G.order, &G.ck,
+                  totals_of(B.d_err) + g, G.P, &G.keys, &G.vals, &G.ranges, &G.order, &G.ck,
                   &G.n_jobs_bound, for_forward);
     // test_fault 3 (debug builds): the compositors' bound on instance numbers is half the
     // records written, so the entries of the upper half fail the check while every access the
@@ -987,7 +1003,7 @@ void build_group_lists(dgs_ctx* ctx, const Batch& B, int g, ListBufs& lb, cudaSt
 int check_lists(dgs_ctx* ctx, const Batch& B, int g, const GroupLists& G, cudaStream_t s) {
     (void)B;
     uint32_t n = 0;
-    DGS_CUDA(ctx, cudaMemcpyAsync(&n, static_cast<uint32_t*>(ctx->totals.p) + g, sizeof(uint32_t),
+    DGS_CUDA(ctx, cudaMemcpyAsync(&n, totals_of(B.d_err) + g, sizeof(uint32_t),
                                   cudaMemcpyDeviceToHost, s));
     DGS_CUDA(ctx, cudaStreamSynchronize(s));
     n = std::min(n, G.n_bound);
@@ -999,7 +1015,7 @@ int check_lists(dgs_ctx* ctx, const Batch& B, int g, const GroupLists& G, cudaSt
         DGS_CUDA(ctx, cudaMemcpy(vals.data(), G.vals, sizeof(uint32_t) * n, cudaMemcpyDeviceToHost));
     }
     if (!ranges.empty())
-        DGS_CUDA(ctx, cudaMemcpy(ranges.data(), G.lb->ranges.p, sizeof(uint2) * ranges.size(), cudaMemcpyDeviceToHost));
+        DGS_CUDA(ctx, cudaMemcpy(ranges.data(), G.ranges, sizeof(uint2) * ranges.size(), cudaMemcpyDeviceToHost));
     if (!rec.empty())
         DGS_CUDA(ctx, cudaMemcpy(rec.data(), G.lb->records.p, sizeof(Record) * rec.size(), cudaMemcpyDeviceToHost));
     if (ctx->opt.test_fault == 2 && g == 0)
@@ -1064,14 +1080,13 @@ int check_lists(dgs_ctx* ctx, const Batch& B, int g, const GroupLists& G, cudaSt
 
 // Final synchronisation, device error word and kernel times.
 int finish(dgs_ctx* ctx, const Batch& B, cudaStream_t stream) {
-    uint32_t* h_err = reinterpret_cast<uint32_t*>(static_cast<char*>(ctx->h_read) + sizeof(uint64_t) * 2 * (B.V + 1));
-    uint32_t* h_tot = reinterpret_cast<uint32_t*>(static_cast<char*>(ctx->h_read) + sizeof(uint64_t) * 2 * (B.V + 1) + 64);
+    uint32_t* h_blk = reinterpret_cast<uint32_t*>(static_cast<char*>(ctx->h_read) + sizeof(uint64_t) * 2 * (B.V + 1));
     const size_t ng = B.groups.size();
     DGS_CUDA(ctx, cudaGetLastError());
-    DGS_CUDA(ctx, cudaMemcpyAsync(h_err, B.d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, stream));
-    if (ng) DGS_CUDA(ctx, cudaMemcpyAsync(h_tot, ctx->totals.p, sizeof(uint32_t) * ng, cudaMemcpyDeviceToHost, stream));
+    DGS_CUDA(ctx, cudaMemcpyAsync(h_blk, B.d_err, sizeof(uint32_t) * (kTotalsAt + ng), cudaMemcpyDeviceToHost, stream));
     DGS_CUDA(ctx, cudaStreamSynchronize(stream));
-    const uint32_t errw = *h_err;
+    const uint32_t errw = h_blk[0];
+    const uint32_t* h_tot = h_blk + kTotalsAt;
     int64_t pairs = 0;
     for (size_t g = 0; g < ng; ++g) pairs += h_tot[g];
     ctx->stats.n_pairs = pairs;
@@ -1122,7 +1137,7 @@ int run_eager(dgs_ctx* ctx, Batch& B, float* out_rgb, float* out_depth, float* o
         if (ctx->opt.check_binning && (rc = check_lists(ctx, B, g, G, streams[b]))) return rc;
         Launch Lg{streams[b], &ctx->launches};
         tms[b].begin(DGS_K_COMPOSITE);
-        launch_composite(Lg, B.d_views, G.v0, G.v1 - G.v0, G.n_tiles, static_cast<uint2*>(G.lb->ranges.p), G.keys, G.vals,
+        launch_composite(Lg, B.d_views, G.v0, G.v1 - G.v0, G.n_tiles, G.ranges, G.keys, G.vals,
                          static_cast<Record*>(G.lb->records.p), G.P, out_rgb, out_depth, out_alpha, work, G.order,
                          G.ck);
         tms[b].end();
@@ -1214,7 +1229,7 @@ int enqueue_graph_body(dgs_ctx* ctx, const Batch& B, const Launch& L, float* out
                        float* out_alpha) {
     Timer off{ctx, L.stream, false};
     launch_front(ctx, B, L, off);
-    uint32_t* sizes = static_cast<uint32_t*>(ctx->gsizes.p);
+    uint32_t* sizes = sizes_of(B.d_err);
     const int ng = ctx->gng;
     const int vb[3] = {0, ng == 2 ? ctx->gsplit : B.V, B.V};
     GraphGroups G{};
@@ -1248,15 +1263,16 @@ int enqueue_graph_body(dgs_ctx* ctx, const Batch& B, const Launch& L, float* out
         P.view0 = (uint32_t)v0;
         ListBufs& lb = ctx->lists[g];
         const uint32_t *keys = nullptr, *vals = nullptr, *order = nullptr;
+        const uint2* ranges = nullptr;
         Checkpoints ck{};
         uint32_t n_jobs_bound = 0;
         enqueue_lists(ctx, lb, B, Lg, tg, v0, v1, n_tiles, 0u, (uint32_t)ctx->cap_inst[g],
-                      (uint32_t)ctx->cap_pairs[g], sizes + 8 * g, sizes + 8 * g + 3, P, &keys, &vals, &order, &ck,
+                      (uint32_t)ctx->cap_pairs[g], sizes + 8 * g, sizes + 8 * g + 3, P, &keys, &vals, &ranges, &order, &ck,
                       &n_jobs_bound);
-        launch_composite(Lg, B.d_views, v0, v1 - v0, n_tiles, static_cast<uint2*>(lb.ranges.p), keys, vals,
+        launch_composite(Lg, B.d_views, v0, v1 - v0, n_tiles, ranges, keys, vals,
                          static_cast<Record*>(lb.records.p), P, out_rgb, out_depth, out_alpha, nullptr, order, ck);
         ctx->gv0[g] = v0; ctx->gv1[g] = v1; ctx->gtiles[g] = n_tiles;
-        ctx->gkeys[g] = keys; ctx->gvals[g] = vals; ctx->gorder[g] = order; ctx->gP[g] = P;
+        ctx->gkeys[g] = keys; ctx->gvals[g] = vals; ctx->granges[g] = ranges; ctx->gorder[g] = order; ctx->gP[g] = P;
         ctx->gck[g] = ck; ctx->gjobs[g] = n_jobs_bound;
     }
     if (ng == 2) {
@@ -1294,8 +1310,7 @@ int capture_graph(dgs_ctx* ctx, const Batch& B, float* out_rgb, float* out_depth
         if ((rc = ensure_lists(ctx, ctx->lists[g], ctx->cap_inst[g], ctx->cap_pairs[g], n_tiles))) return rc;
     }
     ctx->gbits = bits;
-    if ((rc = ensure(ctx, ctx->gsizes, 128))) return rc;
-    if (!ctx->h_graph) DGS_CUDA(ctx, cudaHostAlloc(&ctx->h_graph, 128, cudaHostAllocDefault));
+    if (!ctx->h_graph) DGS_CUDA(ctx, cudaHostAlloc(&ctx->h_graph, sizeof(uint32_t) * kTotalsAt, cudaHostAllocDefault));
     if (!ctx->cap_stream) DGS_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
     if (!ctx->cap_stream2) DGS_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->cap_stream2, cudaStreamNonBlocking));
     sort_prepare();
@@ -1343,14 +1358,13 @@ int render_graph(dgs_ctx* ctx, Batch& B, float* out_rgb, float* out_depth, float
         }
         ctx->launches = ctx->glaunches;
         char* hg = static_cast<char*>(ctx->h_graph);
-        DGS_CUDA(ctx, cudaMemcpyAsync(hg, ctx->gsizes.p, 96, cudaMemcpyDeviceToHost, stream));
-        DGS_CUDA(ctx, cudaMemcpyAsync(hg + 96, B.d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, stream));
+        DGS_CUDA(ctx, cudaMemcpyAsync(hg, B.d_err, sizeof(uint32_t) * kTotalsAt, cudaMemcpyDeviceToHost, stream));
         DGS_CUDA(ctx, cudaStreamSynchronize(stream));
         uint32_t errw, sizes[16];
         uint64_t raw[4];
-        std::memcpy(sizes, hg, 64);
-        std::memcpy(raw, hg + 64, 32);
-        std::memcpy(&errw, hg + 96, 4);
+        std::memcpy(&errw, hg, 4);
+        std::memcpy(sizes, hg + 4 * kSizesAt, 64);
+        std::memcpy(raw, hg + 4 * kSizesAt + 64, 32);
         if (ctx->opt.profile)
             for (const TimedRange& r : ctx->ranges_timed) {
                 float ms = 0.f;
@@ -1373,7 +1387,7 @@ int render_graph(dgs_ctx* ctx, Batch& B, float* out_rgb, float* out_depth, float
                 G.v0 = ctx->gv0[g]; G.v1 = ctx->gv1[g]; G.n_tiles = ctx->gtiles[g];
                 G.n_bound = (uint32_t)ctx->cap_pairs[g];
                 G.n_inst = (uint32_t)raw[2 * g];      // the replay's live count (at most the capacity)
-                G.keys = ctx->gkeys[g]; G.vals = ctx->gvals[g]; G.order = ctx->gorder[g];
+                G.keys = ctx->gkeys[g]; G.vals = ctx->gvals[g]; G.ranges = ctx->granges[g]; G.order = ctx->gorder[g];
                 G.ck = ctx->gck[g]; G.n_jobs_bound = ctx->gjobs[g];
                 G.lb = &ctx->lists[g];
                 G.P = ctx->gP[g];
@@ -1454,7 +1468,7 @@ int dgs_context_destroy(dgs_ctx* ctx) {
     if (!ctx) return DGS_OK;
     cudaDeviceSynchronize();
     DevBuf* bufs[] = {&ctx->meta, &ctx->counts, &ctx->inst_off, &ctx->pair_off, &ctx->parts, &ctx->errword,
-                      &ctx->readback, &ctx->inst_grad, &ctx->gsizes, &ctx->totals};
+                      &ctx->readback, &ctx->inst_grad};
     for (DevBuf* b : bufs) free_buf(*b);
     for (ListBufs& lb : ctx->lists)
         for (DevBuf* b : lb.all) free_buf(*b);
@@ -1469,6 +1483,7 @@ int dgs_context_destroy(dgs_ctx* ctx) {
     free_buf(ctx->tsdf_meta);
     free_buf(ctx->tsdf_depth);
     if (ctx->h_tsdf) cudaFreeHost(ctx->h_tsdf);
+    if (ctx->meta_copied) cudaEventDestroy(ctx->meta_copied);
     if (ctx->tsdf_copied) cudaEventDestroy(ctx->tsdf_copied);
     for (DevBuf* b : {&ctx->lid_rec, &ctx->lid_box, &ctx->lid_tab, &ctx->lid_meta, &ctx->lid_slots}) free_buf(*b);
     if (ctx->h_lid) cudaFreeHost(ctx->h_lid);
@@ -1484,7 +1499,7 @@ const char* dgs_last_error(const dgs_ctx* ctx) { return ctx ? ctx->err.c_str() :
 int dgs_workspace_query(const dgs_ctx* ctx, size_t* bytes) {
     if (!ctx || !bytes) return DGS_ERR_INVALID_ARG;
     const DevBuf* bufs[] = {&ctx->meta, &ctx->counts, &ctx->inst_off, &ctx->pair_off, &ctx->parts, &ctx->errword,
-                            &ctx->readback, &ctx->inst_grad, &ctx->gsizes, &ctx->totals, &ctx->aug_dev,
+                            &ctx->readback, &ctx->inst_grad, &ctx->aug_dev,
                             &ctx->lid_rec, &ctx->lid_box, &ctx->lid_tab, &ctx->lid_meta, &ctx->lid_slots,
                             &ctx->tsdf_meta, &ctx->tsdf_depth};
     size_t s = 0;
@@ -1648,7 +1663,7 @@ int enqueue_adjoint(dgs_ctx* ctx, const Batch& B, const GroupLists& G, const flo
     Launch L{stream, &ctx->launches};
     tm.begin(DGS_K_BACKWARD);
     DGS_CUDA(ctx, cudaMemsetAsync(ctx->inst_grad.p, 0, sizeof(float) * kInstGrad * std::max<uint32_t>(G.n_inst, 1), stream));
-    launch_composite_bwd(L, B.d_views, G.v0, G.v1 - G.v0, G.n_tiles, static_cast<uint2*>(G.lb->ranges.p), G.keys, G.vals,
+    launch_composite_bwd(L, B.d_views, G.v0, G.v1 - G.v0, G.n_tiles, G.ranges, G.keys, G.vals,
                          static_cast<Record*>(G.lb->records.p), G.P, out_rgb, out_depth, grad_rgb, grad_depth,
                          static_cast<float*>(ctx->inst_grad.p), n_red, G.order, G.ck, G.n_jobs_bound);
     tm.end();
@@ -1697,6 +1712,7 @@ int dgs_render_backward(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nodes, co
         if (grads) std::memcpy(hm, grads, bytes);
         else std::memset(hm, 0, bytes);
         DGS_CUDA(ctx, cudaMemcpyAsync(const_cast<dgs_node_grads*>(B.d_grads), hm, bytes, cudaMemcpyHostToDevice, stream));
+        DGS_CUDA(ctx, cudaEventRecord(ctx->meta_copied, stream));
         DGS_CUDA(ctx, cudaMemsetAsync(B.d_err, 0, kErrBlockBytes, stream));
     } else {
         rc = prepare(ctx, nodes, n_nodes, env_node_ids, n_envs, max_nodes, node_poses, cams, cams_per_env, max_cams,

@@ -6,6 +6,8 @@
 // counts taken in sorted order) and written by walking the instance's tile rectangle with the
 // same exact test that counted them.  A stable sort by tile then leaves every tile's run in
 // depth order, equal depths in emission (id) order.
+#include <algorithm>
+
 #include "dgs_internal.cuh"
 
 namespace dgs {
@@ -16,89 +18,29 @@ constexpr int kPairWarps = 4;
 
 __device__ __forceinline__ uint32_t live(uint32_t n, const uint32_t* d_n) { return d_n ? min(n, *d_n) : n; }
 
-__device__ __forceinline__ uint32_t block_sum(uint32_t x) {
-    __shared__ uint32_t s[kScanThreads / 32];
-    x = __reduce_add_sync(0xffffffffu, x);
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = x;
-    __syncthreads();
-    uint32_t t = 0;
-    for (int w = 0; w < kScanThreads / 32; ++w) t += s[w];
-    return t;
-}
-
-// parts[b] = sum of ntile[order[i]] over partition b
-__global__ void __launch_bounds__(kScanThreads) k_tscan_partial(const uint32_t* __restrict__ order,
-                                                               const uint32_t* __restrict__ ntile, uint32_t n,
-                                                               const uint32_t* __restrict__ d_n, uint32_t* parts,
-                                                               uint32_t* err) {
-    if (sort_failed(err)) return;
-    n = live(n, d_n);
-    const uint32_t base = blockIdx.x * (uint32_t)kScanTile;
-    if (base >= n) return;
-    uint32_t s = 0;
-#pragma unroll
-    for (int j = 0; j < kScanItems; ++j) {
-        const uint32_t i = base + j * kScanThreads + threadIdx.x;
-        if (i < n) {
-            const uint32_t r = order[i];
-            if (in_bounds(r, n, err, kSiteScanInstance)) s += ntile[r];
-        }
-    }
-    s = block_sum(s);
-    if (threadIdx.x == 0) parts[blockIdx.x] = s;
-}
-
-// one block: exclusive scan of the live partitions' sums in place; poff[n] = the grand total
-// and *total = min(grand total, cap)
-__global__ void __launch_bounds__(kScanThreads) k_tscan_parts(uint32_t* parts, uint32_t n, const uint32_t* __restrict__ d_n,
-                                                              uint32_t* poff, uint32_t cap, uint32_t* total) {
+// poff[i] for i <= n and *total in one pass: a block takes the next kScanTile instances from a
+// counter, gathers their counts, publishes their sum and finds the sum of the partitions before it
+// by decoupled look-back (warp 0, 32 predecessors at a time; bounded like the sort's).  Against a
+// pass of partition sums, one block over them and a second gathering pass: 187k instances 18 -> 11 us,
+// 10M 67 -> 69 us (there bound by the gather).
+__global__ void __launch_bounds__(kScanThreads) k_tscan(const uint32_t* __restrict__ order,
+                                                       const uint32_t* __restrict__ ntile, uint32_t n,
+                                                       const uint32_t* __restrict__ d_n, uint32_t* __restrict__ poff,
+                                                       uint32_t* status, uint32_t* counter, uint32_t cap,
+                                                       uint32_t* total, uint32_t* err, uint64_t spin_ns) {
     __shared__ uint32_t s_w[kScanThreads / 32];
-    n = live(n, d_n);
-    const uint32_t np = (n + kScanTile - 1) / kScanTile;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t carry = 0;
-    for (uint32_t b0 = 0; b0 < np; b0 += kScanThreads) {
-        const uint32_t i = b0 + threadIdx.x;
-        const uint32_t x = i < np ? parts[i] : 0u;
-        uint32_t y = x;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(0xffffffffu, y, o);
-            if (lane >= o) y += t;
-        }
-        if (lane == 31) s_w[warp] = y;
-        __syncthreads();
-        uint32_t wpre = 0, all = 0;
-        for (int w = 0; w < kScanThreads / 32; ++w) {
-            if (w < warp) wpre += s_w[w];
-            all += s_w[w];
-        }
-        if (i < np) parts[i] = carry + wpre + y - x;
-        carry += all;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        poff[n] = carry;
-        *total = min(carry, cap);
-    }
-}
-
-// poff[i] for i < n: thread t of block b scans the 16 consecutive entries from 16 t of its tile
-__global__ void __launch_bounds__(kScanThreads) k_tscan_final(const uint32_t* __restrict__ order,
-                                                             const uint32_t* __restrict__ ntile, uint32_t n,
-                                                             const uint32_t* __restrict__ d_n,
-                                                             const uint32_t* __restrict__ parts, uint32_t* poff,
-                                                             uint32_t* err) {
-    __shared__ uint32_t s_w[kScanThreads / 32];
+    __shared__ uint32_t s_part, s_excl;
     // the counts of the block's kScanTile instances, gathered warp-striped (coalesced order
     // reads) into shared memory, one pad word per 16 against bank conflicts; each thread then
     // scans its kScanItems consecutive counts, and the offsets go back the same way
     __shared__ uint32_t s_v[kScanTile + kScanTile / 16];
     auto slot = [](int k) { return k + (k >> 4); };
-    if (sort_failed(err)) return;
+    if (__syncthreads_or(sort_failed(err))) return;
+    if (threadIdx.x == 0) s_part = atomicAdd(counter, 1u);
+    __syncthreads();
+    const uint32_t part = s_part, base = part * (uint32_t)kScanTile;
     n = live(n, d_n);
-    const uint32_t base = blockIdx.x * (uint32_t)kScanTile;
-    if (base >= n) return;
+    if (base >= n && part > 0) return;
 #pragma unroll 4
     for (int j = 0; j < kScanItems; ++j) {
         const int k = j * kScanThreads + threadIdx.x;
@@ -125,8 +67,46 @@ __global__ void __launch_bounds__(kScanThreads) k_tscan_final(const uint32_t* __
     }
     if (lane == 31) s_w[warp] = y;
     __syncthreads();
-    uint32_t run = parts[blockIdx.x] + y - sum;
-    for (int w = 0; w < warp; ++w) run += s_w[w];
+    uint32_t pre = y - sum, all = 0;
+    for (int w = 0; w < kScanThreads / 32; ++w) {
+        if (w < warp) pre += s_w[w];
+        all += s_w[w];
+    }
+    if (warp == 0) {
+        uint32_t excl = 0;
+        if (lane == 0) st_relaxed(&status[part], (part == 0 ? kFlagInc : kFlagAgg) | all);
+        if (part > 0) {
+            int64_t p = (int64_t)part - 1;              // the last predecessor not yet summed
+            uint64_t t0 = 0;
+            uint32_t spins = 0;
+            for (;;) {
+                const uint32_t sv = p - lane >= 0 ? ld_relaxed(&status[p - lane]) : kFlagInc;
+                const uint32_t f = sv & ~kCountMask;
+                const uint32_t inc = __ballot_sync(0xffffffffu, f == kFlagInc), none = __ballot_sync(0xffffffffu, f == 0);
+                const int last = inc ? __ffs(inc) - 1 : 31;   // the predecessors up to here are summed
+                if ((none & ((2u << last) - 1u)) == 0) {
+                    excl += __reduce_add_sync(0xffffffffu, lane <= last ? sv & kCountMask : 0u);
+                    if (inc) break;
+                    p -= 32;
+                    continue;
+                }
+                bool expired = false;
+                if ((++spins & 255u) == 0) {
+                    const uint64_t now = global_timer_ns();
+                    if (t0 == 0) t0 = now;
+                    else expired = now - t0 > spin_ns;
+                }
+                if (__any_sync(0xffffffffu, expired)) {
+                    if (lane == 0) atomicOr(err, kErrTimeout);
+                    break;
+                }
+            }
+            if (lane == 0) st_relaxed(&status[part], kFlagInc | ((excl + all) & kCountMask));
+        }
+        if (lane == 0) s_excl = excl;
+    }
+    __syncthreads();
+    uint32_t run = s_excl + pre;
 #pragma unroll
     for (int j = 0; j < kScanItems; ++j) {
         s_v[slot(threadIdx.x * kScanItems + j)] = run;
@@ -137,6 +117,10 @@ __global__ void __launch_bounds__(kScanThreads) k_tscan_final(const uint32_t* __
     for (int j = 0; j < kScanItems; ++j) {
         const int k = j * kScanThreads + threadIdx.x;
         if (base + k < n) poff[base + k] = s_v[slot(k)];
+    }
+    if (threadIdx.x == 0 && base + (uint32_t)kScanTile >= n) {   // the last partition
+        poff[n] = s_excl + all;
+        *total = min(s_excl + all, cap);
     }
 }
 
@@ -297,15 +281,38 @@ __global__ void __launch_bounds__(kPairWarps * 32) k_pairs(const ViewDesc* __res
 
 }  // namespace
 
-size_t tile_scan_parts(uint32_t n) { return ((size_t)n + kScanTile - 1) / kScanTile + 1; }
+size_t tile_scan_words(uint32_t n) { return (((size_t)n + kScanTile - 1) / kScanTile + 2 + 3) & ~size_t(3); }
 
 void launch_tile_scan(const Launch& L, const uint32_t* order, const uint32_t* ntile, uint32_t n, const uint32_t* d_n,
-                      uint32_t* poff, uint32_t* parts, uint32_t cap, uint32_t* total, uint32_t* err) {
-    const uint32_t blocks = (n + kScanTile - 1) / kScanTile;
-    if (blocks) k_tscan_partial<<<blocks, kScanThreads, 0, L.stream>>>(order, ntile, n, d_n, parts, err);
-    k_tscan_parts<<<1, kScanThreads, 0, L.stream>>>(parts, n, d_n, poff, cap, total);
-    if (blocks) k_tscan_final<<<blocks, kScanThreads, 0, L.stream>>>(order, ntile, n, d_n, parts, poff, err);
-    *L.launches += blocks ? 3 : 1;
+                      uint32_t* poff, uint32_t* scratch, uint32_t cap, uint32_t* total, uint32_t* err,
+                      uint64_t spin_ns) {
+    const uint32_t blocks = n ? (n + kScanTile - 1) / kScanTile : 1u;
+    k_tscan<<<blocks, kScanThreads, 0, L.stream>>>(order, ntile, n, d_n, poff, scratch + 1, scratch, cap, total, err,
+                                                   spin_ns);
+    ++*L.launches;
+}
+
+ListPlan plan_lists(uint32_t n_inst, uint32_t n_pairs, int n_views, int tbits, int64_t n_tiles, bool separate_view_key) {
+    ListPlan p;
+    int vb = 0;
+    while (vb < 31 && (1ll << vb) < n_views) ++vb;
+    if (kZBits + vb <= 32 && !separate_view_key) p.depth_bits = kZBits + vb;
+    else p.view_bits = vb;
+    size_t at = 0;
+    auto take = [&](size_t words) { const size_t r = at; at += (words + 3) & ~size_t(3); return r; };
+    p.depth = take(sort_scratch_words(n_inst, p.depth_bits, p.view_bits));
+    p.tscan = take(tile_scan_words(n_inst));
+    p.tile = take(sort_scratch_words(n_pairs, tbits, 0));
+    p.order = take(kOrderWords);
+    p.ranges = take(2 * (size_t)std::max<int64_t>(n_tiles, 1));
+    p.words = at;
+    return p;
+}
+
+size_t list_scratch_bound(uint32_t n_inst, uint32_t n_pairs, int64_t n_tiles) {
+    // a depth key of 32 bits and a view key of 24, four and three passes of the widest digit
+    return sort_scratch_words(n_inst, 32, 24) + tile_scan_words(n_inst) + sort_scratch_words(n_pairs, kTileBits, 0) +
+           kOrderWords + 2 * (size_t)std::max<int64_t>(n_tiles, 1) + 16;
 }
 
 void launch_pairs(const Launch& L, const ViewDesc* views, int K, const uint32_t* order, const uint32_t* poff,

@@ -89,6 +89,54 @@ __global__ void __launch_bounds__(1024) k_tile_order(const uint2* __restrict__ r
     for (int t = threadIdx.x; t < n_tiles; t += blockDim.x) order[atomicAdd(&cnt[length_bucket(ranges[t])], 1u)] = t;
 }
 
+// The same order for more than kOrderOneBlock tiles, over many blocks: bucket counts, which the last
+// block to finish turns into the buckets' first places, then the placement (28,800 tiles: 16 us,
+// one block takes 26).
+__global__ void __launch_bounds__(256) k_order_count(const uint2* __restrict__ ranges, int n_tiles, uint32_t* cnt, uint32_t* done) {
+    __shared__ uint32_t s_cnt[256];
+    __shared__ bool s_last;
+    __shared__ uint32_t s_w[8];
+    s_cnt[threadIdx.x] = 0;
+    __syncthreads();
+    for (int t = blockIdx.x * 256 + threadIdx.x; t < n_tiles; t += gridDim.x * 256) atomicAdd(&s_cnt[length_bucket(ranges[t])], 1u);
+    __syncthreads();
+    if (s_cnt[threadIdx.x]) atomicAdd(cnt + threadIdx.x, s_cnt[threadIdx.x]);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t v = __ldcg(cnt + threadIdx.x);
+    uint32_t y = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, y, o);
+        if (lane >= o) y += t;
+    }
+    if (lane == 31) s_w[warp] = y;
+    __syncthreads();
+    uint32_t pre = y - v;
+    for (int w = 0; w < warp; ++w) pre += s_w[w];
+    cnt[threadIdx.x] = pre;
+}
+
+__global__ void __launch_bounds__(256) k_order_place(const uint2* __restrict__ ranges, int n_tiles, uint32_t* cnt,
+                                                     uint32_t* __restrict__ order) {
+    __shared__ uint32_t s_cnt[256], s_base[256];
+    s_cnt[threadIdx.x] = 0;
+    __syncthreads();
+    const int t = blockIdx.x * 256 + threadIdx.x;
+    const uint32_t b = t < n_tiles ? length_bucket(ranges[t]) : 0u;
+    const uint32_t rank = t < n_tiles ? atomicAdd(&s_cnt[b], 1u) : 0u;
+    __syncthreads();
+    const uint32_t c = s_cnt[threadIdx.x];          // one global addition per bucket and block
+    if (c) s_base[threadIdx.x] = atomicAdd(cnt + threadIdx.x, c);
+    __syncthreads();
+    if (t < n_tiles) order[s_base[b] + rank] = (uint32_t)t;
+}
+
 // One block: every tile's first checkpoint slot (an exclusive scan of its segments after the
 // first, in tile order), then the (tile, segment) jobs of the adjoint in descending order of
 // their length, bucketed as above; *n_jobs = their number.
@@ -361,7 +409,6 @@ __global__ void __launch_bounds__(kCompWarps * 32, 16) k_composite(const ViewDes
 
 void launch_ranges(const Launch& L, const uint32_t* keys, uint32_t n, uint2* ranges, int n_tiles,
                    const uint32_t* d_n, const ViewDesc* views, int nv, const Params& P) {
-    cudaMemsetAsync(ranges, 0, sizeof(uint2) * (size_t)n_tiles, L.stream);
     if (n == 0) return;
     const uint32_t threads = (n + 3) / 4;
     const uint32_t blocks = std::min<uint32_t>((threads + 255) / 256, sm_count() * 8u);
@@ -370,10 +417,17 @@ void launch_ranges(const Launch& L, const uint32_t* keys, uint32_t n, uint2* ran
     ++*L.launches;
 }
 
-void launch_tile_order(const Launch& L, const uint2* ranges, int n_tiles, uint32_t* order) {
+void launch_tile_order(const Launch& L, const uint2* ranges, int n_tiles, uint32_t* order, uint32_t* scratch) {
     if (n_tiles == 0) return;
-    k_tile_order<<<1, 1024, 0, L.stream>>>(ranges, n_tiles, order);
-    ++*L.launches;
+    if (n_tiles <= kOrderOneBlock) {
+        k_tile_order<<<1, 1024, 0, L.stream>>>(ranges, n_tiles, order);
+        ++*L.launches;
+        return;
+    }
+    const unsigned blocks = (unsigned)((n_tiles + 255) / 256);
+    k_order_count<<<blocks, 256, 0, L.stream>>>(ranges, n_tiles, scratch, scratch + 256);
+    k_order_place<<<blocks, 256, 0, L.stream>>>(ranges, n_tiles, scratch, order);
+    *L.launches += 2;
 }
 
 void launch_segment_jobs(const Launch& L, const uint2* ranges, int n_tiles, const Checkpoints& ck) {

@@ -158,6 +158,7 @@ struct Params {
     uint32_t view0;       // first view of the current view group
     int32_t tbits;        // bits of a tile within its view (tile keys: view in group << tbits | tile)
     int32_t vshift;       // > 0: emission writes instance numbers as r | view in group << vshift
+    int32_t vkey;         // != 0: emission writes depth keys as depth | view in group << kZBits
     const uint32_t* inst_base_dev;  // emission: first record of the group read on the device (graph replay)
     // image randomisation of the RGB output (null aug = none): per-view records, overlay clip
     const dgs_augment* aug;
@@ -417,6 +418,19 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
     return t;
 }
 
+// Decoupled look-back (the sorts and the tile-count scan): a partition's status word is a 2-bit flag
+// (0: nothing yet, aggregate, inclusive prefix) above a 30-bit count.
+constexpr uint32_t kFlagAgg = 1u << 30, kFlagInc = 2u << 30, kCountMask = (1u << 30) - 1u;
+__device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+
 // ------------------------------------------------------------------ launchers (host side)
 struct Launch {
     cudaStream_t stream;
@@ -471,20 +485,40 @@ struct ViewKey {
 // are sized for.  *keys_out / *vals_out receive the buffers holding the result.  A look-back
 // wait that runs out sets kErrTimeout in err (the output is then invalid).  With vk (bits > 0)
 // the values are then sorted stably by their view, as a more significant key; no sorted keys
-// are then written (*keys_out is null).
+// are then written (*keys_out is null).  scratch: sort_scratch_words(n, key_bits, vk ? vk->bits : 0)
+// words, zero on entry.
+size_t sort_scratch_words(uint32_t n, int key_bits, int view_bits);
 void launch_sort(const Launch& L, uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt,
-                 uint32_t n, int key_bits, uint32_t* hist, uint32_t* status, uint32_t* counters, uint32_t* err,
-                 uint32_t** keys_out, uint32_t** vals_out, const uint32_t* d_n = nullptr, SortCtl ctl = SortCtl{},
+                 uint32_t n, int key_bits, uint32_t* scratch, uint32_t* err, uint32_t** keys_out,
+                 uint32_t** vals_out, const uint32_t* d_n = nullptr, SortCtl ctl = SortCtl{},
                  const ViewKey* vk = nullptr);
 
 // Sets the sort kernels' launch attributes; call before a stream capture that contains a sort.
 void sort_prepare();
 
 // K3b: pair offsets in depth order, poff[i] = sum_{j<i} ntile[order[j]] for i <= n (n =
-// min(*d_n, n) if d_n), and *total = min(poff[n], cap).  parts: scratch of
-// tile_scan_parts(n) words.
+// min(*d_n, n) if d_n), and *total = min(poff[n], cap).  scratch: tile_scan_words(n) words, zero on
+// entry.
+size_t tile_scan_words(uint32_t n);
 void launch_tile_scan(const Launch& L, const uint32_t* order, const uint32_t* ntile, uint32_t n, const uint32_t* d_n,
-                      uint32_t* poff, uint32_t* parts, uint32_t cap, uint32_t* total, uint32_t* err);
+                      uint32_t* poff, uint32_t* scratch, uint32_t cap, uint32_t* total, uint32_t* err,
+                      uint64_t spin_ns);
+
+// How a group's lists are keyed and where their parts of one region of words, zeroed at once
+// before the group's kernels, lie: the depth sort's scratch, the tile-count scan's, the tile
+// sort's, the tile order's counters, and the ranges.  The depth key takes the view of the instance
+// above its kZBits bits where both fit in 32: four passes either way, of wider digits (187k instances of
+// two views: 47 us against 41 and 14 for the pass, histogram and scan of a separate key).  Else
+// (view_bits > 0) the view is a key of its own, packed into the instance numbers where those fit in
+// 32 bits together and gathered where not.
+struct ListPlan {
+    int depth_bits = kZBits;            // key bits of the depth sort
+    int view_bits = 0;                  // bits of a separate view key
+    size_t depth = 0, tscan = 0, tile = 0, order = 0, ranges = 0, words = 0;
+};
+ListPlan plan_lists(uint32_t n_inst, uint32_t n_pairs, int n_views, int tbits, int64_t n_tiles, bool separate_view_key);
+// Words that hold the plan of any group of at most these sizes, whatever its views and tile bits.
+size_t list_scratch_bound(uint32_t n_inst, uint32_t n_pairs, int64_t n_tiles);
 
 // Kernels that read sorted values as indices return at once after a sort timed out (the
 // sorted arrays are then not permutations).
@@ -504,7 +538,6 @@ __device__ __forceinline__ bool in_bounds(uint64_t i, uint64_t n, uint32_t* err,
 }
 
 __device__ __forceinline__ bool sort_failed(const uint32_t* err) { return (*(volatile const uint32_t*)err & kErrTimeout) != 0; }
-size_t tile_scan_parts(uint32_t n);
 
 // K3c: the (tile, instance) pairs of the depth-ordered instances, instance by instance in
 // that order and each instance's tiles in row-major order: keys = tile within the group (bits
@@ -519,6 +552,7 @@ void launch_pairs(const Launch& L, const ViewDesc* views, int K, const uint32_t*
 // K4: ranges[tile of the group] = [first, last) entry of its run.  Keys are view in group <<
 // P.tbits | tile in its view (bits 0..23); a key whose view is not below nv (dead pairs) has no
 // tile.
+// ranges is zero on entry (empty tiles stay so).
 void launch_ranges(const Launch& L, const uint32_t* keys, uint32_t n, uint2* ranges, int n_tiles,
                    const uint32_t* d_n, const ViewDesc* views, int nv, const Params& P);
 
@@ -556,10 +590,12 @@ void launch_segment_jobs(const Launch& L, const uint2* ranges, int n_tiles, cons
 // groups of at most kOrderMaxTiles tiles: with more, the many waves of blocks balance the SMs
 // without it.
 constexpr int kOrderMaxTiles = 32768;
+constexpr int kOrderOneBlock = 4096;    // tiles up to which one block orders them
+constexpr size_t kOrderWords = 256 + 4;  // zeroed scratch of the others: bucket counts, then a counter
 // Warps per compositor block (forward and adjoint): each warp one 8x4 sub-tile of the block's
 // tile; a tile of tile_w x tile_h pixels spans tile_w * tile_h / (32 kCompWarps) blocks.
 constexpr int kCompWarps = 2;
-void launch_tile_order(const Launch& L, const uint2* ranges, int n_tiles, uint32_t* order);
+void launch_tile_order(const Launch& L, const uint2* ranges, int n_tiles, uint32_t* order, uint32_t* scratch);
 
 // Image randomisation of an RGB batch in place (the separate form of the compositor's
 // epilogue).  spans[V]: per view its first output pixel, its first quad in the view-by-view
@@ -652,7 +688,6 @@ void launch_project_bwd(const Launch& L, int dtype_mask, const NodeDesc* nodes, 
 // se(3) twists (rho, phi) [n,6] of n poses [n,12] and their 3x4 gradients [n,12].
 void launch_pose_twist(const Launch& L, const float* poses, const float* grads, int64_t n, float* out);
 
-size_t sort_status_words(uint32_t n);
 int sort_passes(int key_bits);
 // Streaming multiprocessors of the current device (read once per process and device).
 uint32_t sm_count();

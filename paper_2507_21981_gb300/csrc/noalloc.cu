@@ -171,18 +171,12 @@ extern "C" int dgs_render_noalloc(const dgs_options* opt, const dgs_node* nodes,
     uint32_t* d_dk1 = cv.take<uint32_t>(ni);
     uint32_t* d_iv1 = cv.take<uint32_t>(ni);
     uint32_t* d_ntile = cv.take<uint32_t>(ni);
-    uint32_t* d_vig = cv.take<uint32_t>(ni);
     uint32_t* d_poff = cv.take<uint32_t>(ni + 1);
-    uint32_t* d_tparts = cv.take<uint32_t>(tile_scan_parts((uint32_t)ni));
     uint32_t* d_k0 = cv.take<uint32_t>(np);
     uint32_t* d_v0 = cv.take<uint32_t>(np);
     uint32_t* d_k1 = cv.take<uint32_t>(np);
     uint32_t* d_v1 = cv.take<uint32_t>(np);
-    uint32_t* d_hist = cv.take<uint32_t>(8 * 256);
-    uint32_t* d_cnt = cv.take<uint32_t>(8);
     uint32_t* d_total = cv.take<uint32_t>(1);
-    uint32_t* d_status = cv.take<uint32_t>(sort_status_words((uint32_t)std::max(ni, np)));
-    uint2* d_ranges = cv.take<uint2>((size_t)tiles_total);
     if (!cv.ok) return DGS_ERR_CAPACITY;
     // tile keys: view << tbits | tile in view, as in dgs_render with one view group
     int64_t max_view_tiles = 1;
@@ -191,9 +185,16 @@ extern "C" int dgs_render_noalloc(const dgs_options* opt, const dgs_node* nodes,
     if (tbits > kTileBits || tiles_total > kMaxGroupTiles || (int64_t)V >= (1ll << (kTileBits - tbits)))
         return DGS_ERR_CAPACITY;
     // depth-ordered tile lists, as in dgs_render with one view group
-    // the depth sort's view key, packed into the instance numbers where both fit in 32 bits
+    const ListPlan plan = plan_lists((uint32_t)n_vis, (uint32_t)n_pairs, V, tbits, tiles_total, false);
+    uint32_t* d_scratch = cv.take<uint32_t>(plan.words);
+    if (!cv.ok) return DGS_ERR_CAPACITY;
+    uint2* d_ranges = reinterpret_cast<uint2*>(d_scratch + plan.ranges);
+    NA_CUDA(cudaMemsetAsync(d_scratch, 0, sizeof(uint32_t) * plan.words, stream));
+    // a separate view key of the depth sort: packed into the instance numbers where both fit in 32
+    // bits, else in the tile sort's second key buffer (pairs are at least as many as instances)
     ViewKey vk;
-    vk.bits = bits_for_tiles((uint64_t)V);
+    vk.bits = plan.view_bits;
+    uint32_t* const d_vig = d_k1;
     if (vk.bits > 0 && bits_for_tiles(n_vis) + vk.bits <= 32) vk.vshift = 32 - vk.bits;
     vk.vig = vk.bits > 0 && !vk.vshift ? d_vig : nullptr;
     vk.inst_off = d_inst_off;
@@ -204,18 +205,20 @@ extern "C" int dgs_render_noalloc(const dgs_options* opt, const dgs_node* nodes,
     P.view0 = 0;
     P.tbits = tbits;
     P.vshift = vk.vshift;
+    P.vkey = plan.depth_bits > kZBits;
     launch_emit(L, dtype_mask, d_nodes, n_nodes, d_views, d_vnodes, K, d_nv, d_nvoff, (int)chunk_total, P, 0, V, true,
                 nullptr, 0, d_counts, d_inst_off, 0u, d_rec, d_info, d_dk0, d_iv0, d_ntile, vk.vig ? d_vig : nullptr);
     uint32_t *dk, *order, *tk, *tv;
     SortCtl depth_ctl;
     depth_ctl.runs = true;
-    launch_sort(L, d_dk0, d_iv0, d_dk1, d_iv1, (uint32_t)n_vis, kZBits, d_hist, d_status, d_cnt, d_err, &dk, &order,
-                nullptr, depth_ctl, &vk);
-    launch_tile_scan(L, order, d_ntile, (uint32_t)n_vis, nullptr, d_poff, d_tparts, (uint32_t)n_pairs, d_total, d_err);
+    launch_sort(L, d_dk0, d_iv0, d_dk1, d_iv1, (uint32_t)n_vis, plan.depth_bits, d_scratch + plan.depth, d_err,
+                &dk, &order, nullptr, depth_ctl, &vk);
+    launch_tile_scan(L, order, d_ntile, (uint32_t)n_vis, nullptr, d_poff, d_scratch + plan.tscan, (uint32_t)n_pairs,
+                     d_total, d_err, depth_ctl.spin_ns);
     launch_pairs(L, d_views, K, order, d_poff, d_rec, d_info, (uint32_t)n_vis, nullptr, P, d_k0, d_v0, (uint32_t)n_pairs);
     SortCtl tile_ctl;
     tile_ctl.runs = true;
-    launch_sort(L, d_k0, d_v0, d_k1, d_v1, (uint32_t)n_pairs, tbits, d_hist, d_status, d_cnt, d_err, &tk, &tv, d_total,
+    launch_sort(L, d_k0, d_v0, d_k1, d_v1, (uint32_t)n_pairs, tbits, d_scratch + plan.tile, d_err, &tk, &tv, d_total,
                 tile_ctl);
     launch_ranges(L, tk, (uint32_t)n_pairs, d_ranges, (int)tiles_total, d_total, d_views, V, P);
     launch_composite(L, d_views, 0, V, (int)tiles_total, d_ranges, tk, tv, d_rec, P, out_rgb, out_depth, out_alpha,

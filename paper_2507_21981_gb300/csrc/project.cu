@@ -549,8 +549,8 @@ __device__ __forceinline__ void process_chunk(const NodeDesc& nd, int c, int lan
                         // projection: a dead record, last in depth order, with no tile pairs
                         out.rec[r] = Record{};
                         out.info[r] = InstInfo{(uint32_t)(nd.gbase + i), (uint32_t)vvj};
-                        out.dkey[r] = (1u << kZBits) - 1u;
                         const uint32_t vg = (uint32_t)vvj / (uint32_t)K - P.view0;
+                        out.dkey[r] = ((1u << kZBits) - 1u) | (P.vkey ? vg << kZBits : 0u);
                         out.ival[r] = P.vshift ? r | vg << P.vshift : r;
                         out.ntile[r] = 0u;
                         if (out.vig) out.vig[r] = vg;
@@ -565,8 +565,8 @@ __device__ __forceinline__ void process_chunk(const NodeDesc& nd, int c, int lan
                         R.r2 = make_float4(rgb[0], rgb[1], rgb[2], __uint_as_float((uint32_t)s.y0 | ((uint32_t)s.y1 << 16)));
                         out.rec[r] = R;
                         out.info[r] = InstInfo{(uint32_t)(nd.gbase + i), (uint32_t)vvj};
-                        out.dkey[r] = min(__float_as_uint(s.z) - P.zbase, (1u << kZBits) - 1u);
                         const uint32_t vg = (uint32_t)vvj / (uint32_t)K - P.view0;
+                        out.dkey[r] = min(__float_as_uint(s.z) - P.zbase, (1u << kZBits) - 1u) | (P.vkey ? vg << kZBits : 0u);
                         out.ival[r] = P.vshift ? r | vg << P.vshift : r;
                         if (out.vig) out.vig[r] = vg;
                         // exact tile pairs: the runs of tiles each tile row's band reaches

@@ -7,7 +7,8 @@
 // order -- by their tile within the view.  Stability carries the depth order, and the id order
 // of equal depths, into every (view, tile) run.
 //
-// Structure: one upfront pass builds the histograms of every digit at once; then each digit is
+// Structure: one upfront pass builds the histograms of every digit at once, its last block to
+// finish turning them into the digits' first places; then each digit is
 // one kernel in which a block takes the next 3072-key partition from an atomic counter, ranks
 // its keys by digit inside the block (per-bit warp ballots + per-warp counters), publishes its
 // digit counts, scatters its keys into shared memory in digit order, and only then finds its
@@ -26,6 +27,7 @@
 // that use sorted values as indices return at once when they see kErrTimeout, and the host
 // reports the timeout.
 #include <algorithm>
+#include <utility>
 
 #include "dgs_internal.cuh"
 
@@ -39,18 +41,8 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kMaxD = 8;                          // widest digit: 256 bins
 constexpr int kMaxR = 1 << kMaxD;
 constexpr int kWindow = 4;                        // predecessors read per digit and look-back round
-constexpr uint32_t kFlagAgg = 1u << 30, kFlagInc = 2u << 30, kCountMask = (1u << 30) - 1u;
 constexpr int kSmem = kTile * 8 + kWarps * kMaxR * 4;
 constexpr int kKeysIn = 0, kKeysGather = 1, kKeysPacked = 2;   // where a pass's key comes from
-
-__device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
-    uint32_t v;
-    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
-    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
 
 __device__ __forceinline__ uint32_t live_count(uint32_t n, const uint32_t* d_n) { return d_n ? min(*d_n, n) : n; }
 
@@ -60,11 +52,49 @@ __device__ __forceinline__ uint32_t live_count(uint32_t n, const uint32_t* d_n) 
 // run of equal digits -- for keys whose high digits repeat over neighbours (tile keys emitted
 // instance by instance, depth keys emitted node chunk by node chunk), whose lanes would
 // otherwise all add to one counter; else a grid-stride loop with one atomic per key and pass.
+// The last block to finish (done: a zeroed counter) replaces every pass's counts by their exclusive
+// scan, and adds the view passes' (VH.passes > 0) from the count scan: view j of the group holds
+// inst_off[view_tab[v0 + j + 1]] - inst_off[view_tab[v0 + j]] instance numbers.
+struct ViewHist {
+    const uint32_t* inst_off = nullptr;
+    const int64_t* view_tab = nullptr;
+    int v0 = 0, nv = 0, passes = 0, D = 0, last_bits = 0;
+};
+
+// Exclusive scans of up to four values per thread over the block, all at once.
+__device__ __forceinline__ void block_excl_scan4(uint32_t (&v)[4]) {
+    __shared__ uint32_t s_w[4][kWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t y[4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) y[p] = v[p];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, y[p], o);
+            if (lane >= o) y[p] += t;
+        }
+    if (lane == 31) {
+#pragma unroll
+        for (int p = 0; p < 4; ++p) s_w[p][warp] = y[p];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        v[p] = y[p] - v[p];
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) v[p] += w < warp ? s_w[p][w] : 0u;
+    }
+    __syncthreads();
+}
+
 template <bool RUNS>
 __global__ void __launch_bounds__(kThreads) k_hist(const uint32_t* __restrict__ keys, uint32_t n,
                                                    const uint32_t* __restrict__ d_n, int passes, int D,
-                                                   int last_bits, uint32_t* hist) {
+                                                   int last_bits, uint32_t* hist, uint32_t* done, ViewHist VH) {
     __shared__ uint32_t sh_all[kWarps][4 * kMaxR];   // one private histogram per warp
+    __shared__ bool s_last;
     uint32_t* sh = sh_all[threadIdx.x >> 5];
     n = live_count(n, d_n);
     // every pass's digit is D bits but the last one's, last_bits (the key bits above are not sorted)
@@ -116,39 +146,40 @@ __global__ void __launch_bounds__(kThreads) k_hist(const uint32_t* __restrict__ 
         for (int w = 0; w < kWarps; ++w) t += sh_all[w][i];
         if (t) atomicAdd(&hist[(i / R) * kMaxR + (i % R)], t);
     }
-}
-
-// one block, 256 threads: exclusive scan of each pass's R bins, in place (4 bins per thread)
-__global__ void __launch_bounds__(256) k_hist_scan(uint32_t* hist, int passes, int R) {
-    __shared__ uint32_t s_w[8];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int p = 0; p < passes; ++p) {
-        uint32_t* h = hist + p * kMaxR;
-        uint32_t v[4], sum = 0;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    static_assert(kMaxR <= kThreads, "one bin per thread");
+    const int b = threadIdx.x;
+    uint32_t x[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int b = threadIdx.x * 4 + j;
-            v[j] = b < R ? h[b] : 0u;
-            sum += v[j];
-        }
-        uint32_t y = sum;
+    for (int p = 0; p < 4; ++p) x[p] = p < passes && b < kMaxR ? __ldcg(hist + p * kMaxR + b) : 0u;   // (bins past the digit's are zero)
+    block_excl_scan4(x);
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(0xffffffffu, y, o);
-            if (lane >= o) y += t;
+    for (int p = 0; p < 4; ++p)
+        if (p < passes && b < kMaxR) hist[p * kMaxR + b] = x[p];
+    if (VH.passes == 0) return;
+    uint32_t* const vh = &sh_all[0][0];
+    for (int i = threadIdx.x; i < VH.passes * kMaxR; i += kThreads) vh[i] = 0;
+    __syncthreads();
+    for (int j = threadIdx.x; j < VH.nv; j += kThreads) {
+        const uint32_t c = VH.inst_off[VH.view_tab[VH.v0 + j + 1]] - VH.inst_off[VH.view_tab[VH.v0 + j]];
+        if (!c) continue;
+        for (int p = 0; p < VH.passes; ++p) {
+            const uint32_t mask = (1u << (p == VH.passes - 1 ? VH.last_bits : VH.D)) - 1u;
+            atomicAdd(&vh[p * kMaxR + (((uint32_t)j >> (VH.D * p)) & mask)], c);
         }
-        if (lane == 31) s_w[warp] = y;
-        __syncthreads();
-        uint32_t run = y - sum;
-        for (int w = 0; w < warp; ++w) run += s_w[w];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int b = threadIdx.x * 4 + j;
-            if (b < R) h[b] = run;
-            run += v[j];
-        }
-        __syncthreads();
     }
+    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < 4; ++p) x[p] = p < VH.passes && b < kMaxR ? vh[p * kMaxR + b] : 0u;
+    block_excl_scan4(x);
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+        if (p < VH.passes && b < kMaxR) hist[(passes + p) * kMaxR + b] = x[p];
 }
 
 // One digit pass.  Thread t owns digits t, t + 256, ... (< 2^D) in the per-digit phases
@@ -367,28 +398,6 @@ OnesweepFn onesweep_for(int D) {
     }
 }
 
-// Histograms of the view passes' digits, from the count scan rather than from the values: view
-// j of the group holds inst_off[view_tab[v0 + j + 1]] - inst_off[view_tab[v0 + j]] instance
-// numbers.  One block; the bins are stored, not added.
-__global__ void __launch_bounds__(kThreads) k_view_hist(const uint32_t* __restrict__ inst_off,
-                                                        const int64_t* __restrict__ view_tab, int v0, int nv,
-                                                        int passes, int D, int last_bits, uint32_t* hist) {
-    __shared__ uint32_t sh[4 * kMaxR];
-    const uint32_t R = 1u << D;
-    for (int i = threadIdx.x; i < passes * (int)R; i += kThreads) sh[i] = 0;
-    __syncthreads();
-    for (int j = threadIdx.x; j < nv; j += kThreads) {
-        const uint32_t c = inst_off[view_tab[v0 + j + 1]] - inst_off[view_tab[v0 + j]];
-        if (!c) continue;
-        for (int p = 0; p < passes; ++p) {
-            const uint32_t mask = p == passes - 1 ? (1u << last_bits) - 1u : R - 1u;
-            atomicAdd(&sh[p * R + (((uint32_t)j >> (D * p)) & mask)], c);
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < passes * (int)R; i += kThreads) hist[(i / R) * kMaxR + (i % R)] = sh[i];
-}
-
 }  // namespace
 
 // Streaming multiprocessors of the current device (read once per process and device).
@@ -405,7 +414,39 @@ uint32_t sm_count() {
 
 int sort_passes(int key_bits) { return std::max(1, (key_bits + kMaxD - 1) / kMaxD); }
 
-size_t sort_status_words(uint32_t n) { return ((size_t)n + kTile - 1) / kTile * kMaxR; }
+namespace {
+
+// Passes of a sort of n keys and the places of its parts in the zeroed scratch: histograms, then
+// counters (one per pass, and the histogram's), then every pass's look-back status.
+struct SortPlan {
+    int passes, D, last, vpasses, vD, vlast;
+    uint32_t parts;
+    size_t counters, status[8], words;
+    SortPlan(uint32_t n, int key_bits, int view_bits) {
+        const int bits = std::max(1, key_bits);
+        passes = sort_passes(bits);
+        D = (bits + passes - 1) / passes;
+        last = bits - D * (passes - 1);               // exactly key_bits bits are sorted
+        vpasses = view_bits > 0 ? sort_passes(view_bits) : 0;
+        vD = vpasses ? (view_bits + vpasses - 1) / vpasses : 0;
+        vlast = vpasses ? view_bits - vD * (vpasses - 1) : 0;
+        parts = (n + kTile - 1) / kTile;
+        counters = (size_t)kMaxR * (passes + vpasses);
+        words = counters + 16;
+        for (int p = 0; p < passes + vpasses; ++p) {
+            status[p] = words;
+            words += (size_t)parts << digit_bits(p);
+        }
+        words = (words + 3) & ~size_t(3);
+    }
+    int digit_bits(int p) const {
+        return p < passes ? (p == passes - 1 ? last : D) : (p - passes == vpasses - 1 ? vlast : vD);
+    }
+};
+
+}  // namespace
+
+size_t sort_scratch_words(uint32_t n, int key_bits, int view_bits) { return SortPlan(n, key_bits, view_bits).words; }
 
 void sort_prepare() {
     static bool attr_set = false;
@@ -419,68 +460,45 @@ void sort_prepare() {
     }
 }
 
-// hist: [8 * 256] words, counters: [8] words, status: sort_status_words(n) words.
 void launch_sort(const Launch& L, uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt, uint32_t n,
-                 int key_bits, uint32_t* hist, uint32_t* status, uint32_t* counters, uint32_t* err,
-                 uint32_t** keys_out, uint32_t** vals_out, const uint32_t* d_n, SortCtl ctl, const ViewKey* vk) {
+                 int key_bits, uint32_t* scratch, uint32_t* err, uint32_t** keys_out, uint32_t** vals_out,
+                 const uint32_t* d_n, SortCtl ctl, const ViewKey* vk) {
     *keys_out = keys;
     *vals_out = vals;
     // with a device-side count every pass runs (the output lands in the same buffer whatever
     // the count); a host-known count of 0 or 1 is already sorted
     if (n <= 1 && !d_n) return;
     if (n == 0) return;
-    const int bits = std::max(1, key_bits);
-    const int passes = sort_passes(bits);
-    const int D = (bits + passes - 1) / passes;
-    const int last_bits = bits - D * (passes - 1);      // exactly key_bits bits are sorted
-    sort_prepare();
-    cudaMemsetAsync(hist, 0, sizeof(uint32_t) * kMaxR * passes, L.stream);
-    cudaMemsetAsync(counters, 0, sizeof(uint32_t) * 8, L.stream);
-    const int hist_blocks = (int)std::min<uint32_t>(4 * sm_count(), (n + kThreads * 8 - 1) / (kThreads * 8));
-    if (ctl.runs) k_hist<true><<<hist_blocks, kThreads, 0, L.stream>>>(keys, n, d_n, passes, D, last_bits, hist);
-    else k_hist<false><<<hist_blocks, kThreads, 0, L.stream>>>(keys, n, d_n, passes, D, last_bits, hist);
-    k_hist_scan<<<1, 256, 0, L.stream>>>(hist, passes, 1 << D);
-    *L.launches += 2;
-    const uint32_t parts = (n + kTile - 1) / kTile;
     const bool by_view = vk && vk->bits > 0;
+    const SortPlan S(n, key_bits, by_view ? vk->bits : 0);
+    sort_prepare();
+    uint32_t* const hist = scratch;
+    uint32_t* const counters = scratch + S.counters;
+    ViewHist VH;
+    if (by_view) VH = ViewHist{vk->inst_off, vk->view_tab, vk->v0, vk->nv, S.vpasses, S.vD, S.vlast};
+    const int hist_blocks = (int)std::min<uint32_t>(4 * sm_count(), (n + kThreads * 8 - 1) / (kThreads * 8));
+    auto* hk = ctl.runs ? k_hist<true> : k_hist<false>;
+    hk<<<hist_blocks, kThreads, 0, L.stream>>>(keys, n, d_n, S.passes, S.D, S.last, hist, counters + 15, VH);
+    ++*L.launches;
     uint32_t *ki = keys, *ko = keys_alt;
     uint32_t *vi = vals, *vo = vals_alt;
-    for (int p = 0; p < passes; ++p) {
-        const int Dp = p == passes - 1 ? last_bits : D;
-        const OnesweepFn fn = onesweep_for<false>(Dp);
-        // the view passes read no keys: the last key pass before them writes none
-        uint32_t* kw = by_view && p == passes - 1 ? nullptr : ko;
-        cudaMemsetAsync(status, 0, sizeof(uint32_t) * (size_t)(1 << Dp) * parts, L.stream);
-        fn<<<parts, kThreads, kSmem, L.stream>>>(ki, vi, kw, vo, n, d_n, D * p, hist + p * kMaxR, status, counters + p,
-                                                 err, ctl.spin_ns, p == 0 ? ctl.mute_part : 0xFFFFFFFFu, nullptr, 0,
-                                                 0xFFFFFFFFu);
+    const bool packed = by_view && vk->vshift > 0;
+    for (int p = 0; p < S.passes + S.vpasses; ++p) {
+        // the last passes' key is the most significant one, the view, derived from the values (their
+        // high bits, stripped by the last pass, or vig[value]); no keys are written for them
+        const bool view = p >= S.passes;
+        const int Dp = S.digit_bits(p), shift = view ? S.vD * (p - S.passes) : S.D * p;
+        const OnesweepFn fn = !view ? onesweep_for<kKeysIn>(Dp) : packed ? onesweep_for<kKeysPacked>(Dp)
+                                                                         : onesweep_for<kKeysGather>(Dp);
+        uint32_t* kw = by_view && p >= S.passes - 1 ? nullptr : ko;
+        const uint32_t vmask = packed && p == S.passes + S.vpasses - 1 ? (1u << vk->vshift) - 1u : 0xFFFFFFFFu;
+        fn<<<S.parts, kThreads, kSmem, L.stream>>>(ki, vi, kw, vo, n, d_n, shift, hist + p * kMaxR,
+                                                   scratch + S.status[p], counters + p, err, ctl.spin_ns,
+                                                   p == 0 ? ctl.mute_part : 0xFFFFFFFFu, view ? vk->vig : nullptr,
+                                                   view ? vk->vshift : 0, vmask);
         ++*L.launches;
-        uint32_t* tk = ki; ki = ko; ko = tk;
-        uint32_t* tv = vi; vi = vo; vo = tv;
-    }
-    // the most significant key, the view, derived from the values (their high bits, or vig[value]);
-    // its histogram comes from the per-view counts of the count scan
-    if (by_view) {
-        const int ip = sort_passes(vk->bits);
-        const int Di = (vk->bits + ip - 1) / ip;
-        const int ilast = vk->bits - Di * (ip - 1);
-        uint32_t* ih = hist + passes * kMaxR;
-        k_view_hist<<<1, kThreads, 0, L.stream>>>(vk->inst_off, vk->view_tab, vk->v0, vk->nv, ip, Di, ilast, ih);
-        k_hist_scan<<<1, 256, 0, L.stream>>>(ih, ip, 1 << Di);
-        *L.launches += 2;
-        const bool packed = vk->vshift > 0;
-        for (int p = 0; p < ip; ++p) {
-            const int Dp = p == ip - 1 ? ilast : Di;
-            const OnesweepFn fi = packed ? onesweep_for<kKeysPacked>(Dp) : onesweep_for<kKeysGather>(Dp);
-            const uint32_t vmask = packed && p == ip - 1 ? (1u << vk->vshift) - 1u : 0xFFFFFFFFu;
-            cudaMemsetAsync(status, 0, sizeof(uint32_t) * (size_t)(1 << Dp) * parts, L.stream);
-            fi<<<parts, kThreads, kSmem, L.stream>>>(ki, vi, ko, vo, n, d_n, Di * p, ih + p * kMaxR, status,
-                                                     counters + passes + p, err, ctl.spin_ns, 0xFFFFFFFFu, vk->vig,
-                                                     vk->vshift, vmask);
-            ++*L.launches;
-            uint32_t* tk = ki; ki = ko; ko = tk;
-            uint32_t* tv = vi; vi = vo; vo = tv;
-        }
+        std::swap(ki, ko);
+        std::swap(vi, vo);
     }
     *keys_out = by_view ? nullptr : ki;
     *vals_out = vi;
