@@ -232,6 +232,25 @@ __device__ __forceinline__ float ld_attr(const void* p, int64_t i) {
     else return __half2float(reinterpret_cast<const __half*>(p)[i]);
 }
 
+// The attributes in 16 bytes, widened: 4 of FP32, 8 of the 16-bit types.
+template <int DT>
+__device__ __forceinline__ void unpack_attr(const uint4& v, float* f) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        if constexpr (DT == DGS_F32) {
+            f[e] = __uint_as_float(w[e]);
+        } else if constexpr (DT == DGS_BF16) {
+            f[2 * e] = __uint_as_float(w[e] << 16);
+            f[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
+        } else {
+            const float2 p = __half22float2(*reinterpret_cast<const __half2*>(&w[e]));
+            f[2 * e] = p.x;
+            f[2 * e + 1] = p.y;
+        }
+    }
+}
+
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31u; }
 
 // Flattened warp walk over the units of up to 32 items.  Items are dense (lane k of the warp

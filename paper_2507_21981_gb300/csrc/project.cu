@@ -431,27 +431,11 @@ __device__ __forceinline__ void stage_sh_n(const NodeDesc& nd, int c, int lane, 
                 for (int j = 0; j < kBatch; ++j) {
                     const int idx = lane + 32 * (i + j), gl = idx / kVec;
                     if (idx >= cnt * kVec) continue;
-                    float* dst = (sh_smem + gl * kShStride + (idx - gl * kVec) * kPer);
-                    const uint32_t w[4] = {v[j].x, v[j].y, v[j].z, v[j].w};
-                    if constexpr (DT == DGS_F32) {
+                    float* dst = sh_smem + gl * kShStride + (idx - gl * kVec) * kPer;
+                    float f[kPer];
+                    unpack_attr<DT>(v[j], f);
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) dst[e] = __uint_as_float(w[e]);
-                    } else {
-                        float f[8];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            if constexpr (DT == DGS_BF16) {
-                                f[2 * e] = __uint_as_float(w[e] << 16);
-                                f[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
-                            } else {
-                                const float2 p = __half22float2(*reinterpret_cast<const __half2*>(&w[e]));
-                                f[2 * e] = p.x;
-                                f[2 * e + 1] = p.y;
-                            }
-                        }
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) dst[e] = f[e];
-                    }
+                    for (int e = 0; e < kPer; ++e) dst[e] = f[e];
                 }
             }
             __syncwarp();
