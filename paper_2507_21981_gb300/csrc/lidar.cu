@@ -168,7 +168,7 @@ __device__ __forceinline__ float slab_enter(const float4 lo, const float4 hi, co
 // Per-warp state in shared memory: the traversal stack (heap index, slot and entry distance of
 // every node still to visit) and the pending hits (bits of t*, global id, alpha), unsorted.
 constexpr int kRayWarps = 4;         // warps (rays in flight) per block
-constexpr int kStack = 256;          // 32 roots + 31 per expansion, at most 6 expansions deep: 218
+constexpr int kStack = 256;          // 32 roots + 31 per expansion, at most 7 expansions deep: 249
 constexpr int kPend = 128;           // pending hits
 constexpr int kPendRegs = kPend / 32;
 constexpr int kKeep = 64;            // hits kept when the pending buffer is cut
@@ -299,10 +299,11 @@ __device__ __forceinline__ uint64_t cut_pending(RayWarp& W, int& cnt, int lane) 
 // sensor are farther apart, at the distances where they hit, than the Gaussians are wide, so
 // neighbouring rays share few leaves: the 32 lanes work on one ray instead, 32 boxes or 32
 // Gaussians per step.
-//   expand   the 2^s (s <= 5) descendants of a node s levels down are consecutive in heap
-//            numbering: one box per lane, one coalesced load; those the ray's interval meets are
-//            pushed nearest on top.  The first expansion of a tree takes the levels that do not
-//            divide by five.
+//   expand   the 2^s (s <= 4) descendants of a node s levels down are consecutive in heap
+//            numbering: one box per lane, one coalesced load; those the ray's interval meets (two
+//            on average) are pushed nearest on top.  Two nodes of a tree on top of the stack are
+//            expanded together, 16 lanes each.  The first expansion of a tree takes the levels
+//            that do not divide by four, so that the last ones before the leaves are full.
 //   leaves   up to four leaves on top of the stack, 8 lanes each: one Gaussian per lane; hits go
 //            to the pending buffer.
 //   flush    a hit is final once its t* lies before the entry of every node still on the stack;
@@ -316,7 +317,7 @@ __device__ __forceinline__ uint64_t cut_pending(RayWarp& W, int& cnt, int lane) 
 // or more warps per SM hide.  Measured against a packet of 32 rays per warp with a 32-hit buffer
 // per lane, same outputs bit for bit: one sensor of 32 x 1024 beams through 380k Gaussians 0.53 ms
 // against 7.4 (there the slowest packet was the time), 16 sensors through 580k 6.0 ms against 28.
-__global__ void __launch_bounds__(kRayWarps * 32) k_lidar_trace(const LidarTreeDev* __restrict__ trees,
+__global__ void __launch_bounds__(kRayWarps * 32, 8) k_lidar_trace(const LidarTreeDev* __restrict__ trees,
                                                                 const LidarSlot* __restrict__ slots, int K,
                                                                 const float* __restrict__ dirs, int n_dirs,
                                                                 int64_t n_rays, LidarParams LP,
@@ -381,13 +382,18 @@ __global__ void __launch_bounds__(kRayWarps * 32) k_lidar_trace(const LidarTreeD
                     levels = 63 - __clzll(tr.P);
                 }
                 if ((int64_t)node < tr.P) {
-                    const int below = levels - (31 - __clz(node));          // levels left to the leaves, >= 1
-                    const int st = below % 5 ? below % 5 : 5;
-                    const uint32_t child = (node << st) + (uint32_t)lane;
-                    --sp;
+                    // the node below on the stack too, if it is an inner one of the same tree
+                    const int at2 = max(sp - 2, 0);
+                    const uint32_t node2 = W.node[at2];
+                    const bool pair = sp >= 2 && W.slot[at2] == slot && (int64_t)node2 < tr.P && W.enter[at2] <= t_hi;
+                    const uint32_t mine = lane >= 16 ? node2 : node;
+                    const int below = levels - (31 - __clz(mine));          // levels left to the leaves, >= 1
+                    const int st = below % 4 ? below % 4 : 4, sub = lane & 15;
+                    const uint32_t child = (mine << st) + (uint32_t)sub;
+                    sp -= pair ? 2 : 1;
                     bool in = false;
                     float en = 0.f;
-                    if (lane < (1 << st)) {
+                    if (sub < (1 << st) && (lane < 16 || pair)) {
                         const float4 lo = __ldg(tr.box + 2 * (size_t)child), hi = __ldg(tr.box + 2 * (size_t)child + 1);
                         in = slab(lo, hi, R.o, R.id, t_lo, t_hi);
                         en = fmaxf(slab_enter(lo, hi, R.o, R.id), t_lo) + 0.f;
