@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(kCompWarps * 32) k_composite_bwd(const ViewDes
                                                g2d.y * (c2d.y - SD));
                         we.y = raw[u] > P.alpha_max ? 0.f : dal * ex[u];
                     }
-                    T = go ? Tn : -fabsf(T);
+                    T = go ? Tn : __int_as_float(__float_as_int(T) | 0x80000000);   // (-|T|)
                     S.we[k + u][lane] = we;
                 }
                 if (__all_sync(0xffffffffu, T < 0.f)) { ended = true; kn = k + kStep; break; }

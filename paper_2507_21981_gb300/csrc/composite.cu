@@ -219,10 +219,9 @@ __global__ void __launch_bounds__(1024) k_segment_jobs(const uint2* __restrict__
 // latency per record; on large batches the shared-memory data path (three 16-byte broadcasts per
 // record move 512 B each to registers: 12 cycles an SM; 88 % busy, 72 % issue).  Measured, one view
 // group, against staging each 32-entry chunk by itself and blending record by record: 64x2
-// 640x480 views 4.15 -> 3.94 ms; 53 ragged views 2.76 -> 1.78; two views 0.145 -> 0.082; one
-// 800x800 view 0.113 -> 0.072 ms.  The packed multiply-adds are 5-10 % of that; kBlend 2 or 8,
-// or 20 blocks (which spills), are slower on the batch; 12 blocks with kBlend 8 are 10 % faster on
-// one view and 4 % slower on the batch.
+// 640x480 views 4.15 -> 3.91 ms; 46 ragged views 2.76 -> 1.73; two views 0.145 -> 0.072.  The
+// packed multiply-adds are 5-10 % of that, marking an ended pixel by its sign bit with an OR
+// 1-2 %; kBlend 2 or 8, or 18 blocks (which spill), are slower on the batch.
 //
 // AUG: the view's image randomisation is applied to the RGB before it is stored.  CK: the
 // per-pixel state is checkpointed at every segment start for the adjoint (see Checkpoints);
@@ -233,8 +232,8 @@ constexpr int kBlend = 4;
 static_assert(kSegEntries % (32 * kScan) == 0, "a scan step must not cross a segment");
 static_assert(kQueue >= 31 + 32 * kScan && (kQueue & (kQueue - 1)) == 0, "ring size");
 
-template <bool COUNT, bool AUG, bool CK>
-__global__ void __launch_bounds__(kCompWarps * 32, 16) k_composite(const ViewDesc* __restrict__ views, int v0, int nv,
+template <bool COUNT, bool AUG, bool CK, int BLOCKS>
+__global__ void __launch_bounds__(kCompWarps * 32, BLOCKS) k_composite(const ViewDesc* __restrict__ views, int v0, int nv,
                                                    const uint2* __restrict__ ranges, const uint32_t* __restrict__ keys,
                                                    const uint32_t* __restrict__ vals,
                                                    const Record* __restrict__ rec, Params P, float* __restrict__ out_rgb,
@@ -377,7 +376,7 @@ __global__ void __launch_bounds__(kCompWarps * 32, 16) k_composite(const ViewDes
                     const float2 c2d = fma2(make_float2(wgt, wgt), make_float2(g2.z, g2.w), make_float2(C2, D));
                     C0 = c01.x; C1 = c01.y; C2 = c2d.x; D = c2d.y;
                 }
-                T = go ? Tn : -fabsf(T);
+                T = go ? Tn : __int_as_float(__float_as_int(T) | 0x80000000);   // (-|T|)
             }
             if (__all_sync(0xffffffffu, T < 0.f)) { n = 0; break; }
         }
@@ -446,9 +445,15 @@ void launch_composite(const Launch& L, const ViewDesc* views, int v0, int n_grou
     if (n_tiles == 0) return;
     // checkpoints are for the adjoint, which never runs on randomised outputs
     const bool with_ck = ck.st != nullptr && !P.aug;
-    auto* kern = with_ck ? (work ? k_composite<true, false, true> : k_composite<false, false, true>)
-                 : work  ? (P.aug ? k_composite<true, true, false> : k_composite<true, false, false>)
-                         : (P.aug ? k_composite<false, true, false> : k_composite<false, false, false>);
+    // few waves: fewer resident blocks with more registers (no spills) shorten the longest lists' chains;
+    // many waves: the most blocks that fit.  One-group times with 14 against 16 blocks an SM: 64 tiles
+    // 16.4 against 18.4 us, 2400 tiles 71.6 / 80, 19200 tiles 268 / 264, 153600 tiles 3986 / 3907.
+    const bool few = n_tiles <= 4096;
+    auto* kern = with_ck ? (work ? k_composite<true, false, true, 16> : few ? k_composite<false, false, true, 14>
+                                                                           : k_composite<false, false, true, 16>)
+                 : work  ? (P.aug ? k_composite<true, true, false, 16> : k_composite<true, false, false, 16>)
+                 : few   ? (P.aug ? k_composite<false, true, false, 14> : k_composite<false, false, false, 14>)
+                         : (P.aug ? k_composite<false, true, false, 16> : k_composite<false, false, false, 16>);
     const int bpt = (P.tile_w * P.tile_h) / (32 * kCompWarps);
     kern<<<n_tiles * bpt, kCompWarps * 32, 0, L.stream>>>(views, v0, n_group_views, ranges, keys, vals, records, P,
                                                           out_rgb, out_depth, out_alpha, work, tile_order, ck);
