@@ -73,7 +73,7 @@ struct dgs_ctx {
     std::unique_ptr<SavedForward> saved;  // valid until the next call stages a batch
     std::string err;
     int device = 0;
-    DevBuf meta, counts, inst_off, pair_off, parts, errword, readback, inst_grad;
+    DevBuf meta, counts, inst_off, pair_off, errword, readback, inst_grad;
     ListBufs lists[2];                    // view groups alternate between two sets (two streams)
     cudaStream_t aux_stream = nullptr;    // second stream of the eager sequence
     uint64_t gen = 0;                     // bumped whenever a workspace buffer is reallocated
@@ -270,7 +270,8 @@ __global__ void k_view_totals(const uint32_t* __restrict__ inst_off, const uint6
 }
 
 // The error word's buffer: the error block, the graph replay's sizes, then the exact pairs of every
-// view group, so that one copy reads a call's results back.
+// view group, so that one copy reads a call's results back; then the count scan's scratch.  One clear
+// at the start of a call covers it.
 constexpr size_t kSizesAt = kErrBlockBytes / 4, kTotalsAt = kSizesAt + 32;   // in words
 uint32_t* sizes_of(uint32_t* err) { return err + kSizesAt; }
 uint32_t* totals_of(uint32_t* err) { return err + kTotalsAt; }
@@ -517,7 +518,9 @@ struct Batch {
     const int64_t* d_vtab = nullptr;
     const int64_t* d_viewtab = nullptr;
     const float* node_poses = nullptr;
-    int64_t n_parts = 0, n_nv = 0;
+    int64_t n_nv = 0;
+    uint32_t* d_scan = nullptr;            // the count scan's scratch
+    size_t call_words = 0;                 // words cleared at the start of a call, from d_err on
     size_t upload_bytes = 0, meta_bytes = 0;
     size_t front_bytes = 0;                // device bytes of the tables up to the count scan
     Params P{};
@@ -607,18 +610,17 @@ int stage(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nodes, const int32_t* e
     const int64_t* d_viewtab = reinterpret_cast<const int64_t*>(dm + o_viewtab);
     VNode* d_vnodes = reinterpret_cast<VNode*>(dm + o_vnodes);
 
-    if ((rc = ensure(ctx, ctx->errword, sizeof(uint32_t) * (kTotalsAt + V + 1)))) return rc;
+    const size_t scan_at = (kTotalsAt + V + 1 + 3) & ~size_t(3), call_words = scan_at + scan_words(T);
+    if ((rc = ensure(ctx, ctx->errword, sizeof(uint32_t) * call_words))) return rc;
     if ((rc = ensure(ctx, ctx->counts, sizeof(uint2) * std::max<int64_t>(T, 1)))) return rc;
     if ((rc = ensure(ctx, ctx->inst_off, sizeof(uint32_t) * (T + 1)))) return rc;
     if ((rc = ensure(ctx, ctx->pair_off, sizeof(uint64_t) * (T + 1)))) return rc;
-    const int64_t n_parts = (T + 4095) / 4096;
-    if ((rc = ensure(ctx, ctx->parts, sizeof(ulonglong2) * (n_parts + 1)))) return rc;
     if ((rc = ensure(ctx, ctx->readback, sizeof(uint64_t) * 2 * (V + 1) + 64))) return rc;
     // pinned: per-view totals, then the error word's buffer
     if ((rc = ensure_host(ctx, ctx->h_read, ctx->h_read_bytes, sizeof(uint64_t) * 2 * (V + 1) + 4 * (kTotalsAt + V + 1))))
         return rc;
-    B.front_bytes = meta_bytes + sizeof(uint32_t) * (kTotalsAt + V + 1) + sizeof(uint2) * std::max<int64_t>(T, 1) + sizeof(uint32_t) * (T + 1) +
-                    sizeof(uint64_t) * (T + 1) + sizeof(ulonglong2) * (n_parts + 1) + sizeof(uint64_t) * 2 * (V + 1) + 64;
+    B.front_bytes = meta_bytes + sizeof(uint32_t) * call_words + sizeof(uint2) * std::max<int64_t>(T, 1) + sizeof(uint32_t) * (T + 1) +
+                    sizeof(uint64_t) * (T + 1) + sizeof(uint64_t) * 2 * (V + 1) + 64;
     uint32_t* d_err = static_cast<uint32_t*>(ctx->errword.p);
 
     DGS_CUDA(ctx, cudaMemcpyAsync(dm, hm, upload_bytes, cudaMemcpyHostToDevice, stream));
@@ -650,16 +652,22 @@ int stage(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nodes, const int32_t* e
     B.P.tbits = tbits;
     B.d_grads = reinterpret_cast<const dgs_node_grads*>(dm + o_grads);
     B.node_poses = node_poses;
-    B.n_parts = n_parts;
+    B.d_scan = d_err + scan_at;
+    B.call_words = call_words;
     B.n_nv = (int64_t)nv.size();
     B.upload_bytes = upload_bytes;
     B.meta_bytes = meta_bytes;
     return DGS_OK;
 }
 
+// Limit of the bounded device waits.
+uint64_t spin_limit_ns(const dgs_options& o) {
+    return o.spin_limit_us > 0 ? (uint64_t)o.spin_limit_us * 1000ull : SortCtl{}.spin_ns;
+}
+
 // Clears the error word, then setup (K0), count (K1) and the exclusive scan of the count table.
 void launch_front(dgs_ctx* ctx, const Batch& B, const Launch& L, Timer& tm) {
-    cudaMemsetAsync(B.d_err, 0, kErrBlockBytes, L.stream);
+    cudaMemsetAsync(B.d_err, 0, sizeof(uint32_t) * B.call_words, L.stream);
     tm.begin(DGS_K_SETUP);
     launch_setup_views(L, B.d_views, B.V, B.node_poses, B.d_slot, B.K, B.d_vnodes, B.d_vtab, B.d_err);
     tm.end();
@@ -675,7 +683,7 @@ void launch_front(dgs_ctx* ctx, const Batch& B, const Launch& L, Timer& tm) {
     }
     tm.end();
     tm.begin(DGS_K_SCAN);
-    launch_scan(L, B.d_counts, B.T, B.d_inst_off, B.d_pair_off, static_cast<ulonglong2*>(ctx->parts.p), B.n_parts + 1);
+    launch_scan(L, B.d_counts, B.T, B.d_inst_off, B.d_pair_off, B.d_scan, B.d_err, spin_limit_ns(ctx->opt));
     tm.end();
 }
 
@@ -732,9 +740,9 @@ int readback_groups(dgs_ctx* ctx, Batch& B, cudaStream_t stream, Timer& tm, size
     tm.begin(DGS_K_SCAN);
     {
         uint64_t* d_rb = static_cast<uint64_t*>(ctx->readback.p);
-        const ulonglong2* scan_total = B.n_parts > 0 ? static_cast<ulonglong2*>(ctx->parts.p) + B.n_parts : nullptr;
+        const ulonglong2* total = B.T > 0 ? scan_total(B.d_scan) : nullptr;
         k_view_totals<<<(V + 1 + 127) / 128, 128, 0, stream>>>(B.d_inst_off, B.d_pair_off, B.d_viewtab, V + 1,
-                                                               scan_total, B.d_err, d_rb);
+                                                               total, B.d_err, d_rb);
         ++ctx->launches;
         DGS_CUDA(ctx, cudaMemcpyAsync(ctx->h_read, d_rb, sizeof(uint64_t) * 2 * (V + 1) + 16, cudaMemcpyDeviceToHost, stream));
     }
@@ -746,6 +754,7 @@ int readback_groups(dgs_ctx* ctx, Batch& B, cudaStream_t stream, Timer& tm, size
     const uint64_t* pair_at = h_rb + (V + 1);
     uint32_t errw = (uint32_t)(h_rb[2 * (V + 1)] & 0xFFFFFFFFu);
     if (errw & kErrPose) return fail(ctx, DGS_ERR_INVALID_ARG, "a node pose is not finite or not rigid");
+    if (errw & kErrTimeout) return fail(ctx, DGS_ERR_TIMEOUT, "a bounded device wait timed out (count scan look-back)");
     const uint64_t n_vis64 = h_rb[2 * (V + 1) + 1];
     ctx->stats.n_visible = (int64_t)n_vis64;
     if (n_vis64 >= (1ull << 32)) return fail(ctx, DGS_ERR_CAPACITY, "2^32 or more visible instances");
@@ -869,7 +878,7 @@ void enqueue_lists(dgs_ctx* ctx, ListBufs& lb, const Batch& B, const Launch& L, 
     tm.begin(DGS_K_SORT);
     uint32_t *dk = nullptr, *order = nullptr;
     SortCtl ctl;
-    if (ctx->opt.spin_limit_us > 0) ctl.spin_ns = (uint64_t)ctx->opt.spin_limit_us * 1000ull;
+    ctl.spin_ns = spin_limit_ns(ctx->opt);
     SortCtl depth_ctl = ctl, tile_ctl = ctl;
     if (ctx->opt.test_fault == 1) depth_ctl.mute_part = 1;
     tile_ctl.runs = true;   // an instance's pairs are consecutive tiles of one view
@@ -1179,6 +1188,7 @@ __global__ void k_graph_sizes(const uint32_t* __restrict__ inst_off, const uint6
     uint64_t ni[2] = {0, 0}, np[2] = {0, 0};
     // the 32-bit instance offsets wrap at 2^32: the scan's 64-bit total decides first
     bool over = G.scan_total && G.scan_total->x >= (1ull << 32);
+    over |= sort_failed(err);                   // the scan gave up waiting: no offset is valid
     for (int g = 0; g < G.ng; ++g) {
         ni[g] = (uint64_t)inst_off[G.t1[g]] - inst_off[G.t0[g]];
         np[g] = pair_off[G.t1[g]] - pair_off[G.t0[g]];
@@ -1234,7 +1244,7 @@ int enqueue_graph_body(dgs_ctx* ctx, const Batch& B, const Launch& L, float* out
     const int vb[3] = {0, ng == 2 ? ctx->gsplit : B.V, B.V};
     GraphGroups G{};
     G.ng = ng;
-    G.scan_total = B.n_parts > 0 ? static_cast<ulonglong2*>(ctx->parts.p) + B.n_parts : nullptr;
+    G.scan_total = B.T > 0 ? scan_total(B.d_scan) : nullptr;
     for (int g = 0; g < ng; ++g) {
         G.t0[g] = B.view_tab[vb[g]];
         G.t1[g] = B.view_tab[vb[g + 1]];
@@ -1467,7 +1477,7 @@ int dgs_set_options(dgs_ctx* ctx, const dgs_options* opt) {
 int dgs_context_destroy(dgs_ctx* ctx) {
     if (!ctx) return DGS_OK;
     cudaDeviceSynchronize();
-    DevBuf* bufs[] = {&ctx->meta, &ctx->counts, &ctx->inst_off, &ctx->pair_off, &ctx->parts, &ctx->errword,
+    DevBuf* bufs[] = {&ctx->meta, &ctx->counts, &ctx->inst_off, &ctx->pair_off, &ctx->errword,
                       &ctx->readback, &ctx->inst_grad};
     for (DevBuf* b : bufs) free_buf(*b);
     for (ListBufs& lb : ctx->lists)
@@ -1498,7 +1508,7 @@ const char* dgs_last_error(const dgs_ctx* ctx) { return ctx ? ctx->err.c_str() :
 
 int dgs_workspace_query(const dgs_ctx* ctx, size_t* bytes) {
     if (!ctx || !bytes) return DGS_ERR_INVALID_ARG;
-    const DevBuf* bufs[] = {&ctx->meta, &ctx->counts, &ctx->inst_off, &ctx->pair_off, &ctx->parts, &ctx->errword,
+    const DevBuf* bufs[] = {&ctx->meta, &ctx->counts, &ctx->inst_off, &ctx->pair_off, &ctx->errword,
                             &ctx->readback, &ctx->inst_grad, &ctx->aug_dev,
                             &ctx->lid_rec, &ctx->lid_box, &ctx->lid_tab, &ctx->lid_meta, &ctx->lid_slots,
                             &ctx->tsdf_meta, &ctx->tsdf_depth};

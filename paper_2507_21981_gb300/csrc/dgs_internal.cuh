@@ -469,8 +469,13 @@ void launch_count(const Launch& L, int dtype_mask, const NodeDesc* nodes, int n_
                   int n_chunks_total, const Params& P, int v0, int v1, bool batched, const int32_t* view_chunk_nodes,
                   int64_t view_chunks, uint2* counts);
 
+// Exclusive scan of the count table: inst_off[n + 1] (32 bits, wrapping), pair_off[n + 1].  scratch:
+// scan_words(n) words, 16-byte aligned and zero on entry; *scan_total(scratch) receives the 64-bit
+// totals (n > 0).
+size_t scan_words(int64_t n);
+ulonglong2* scan_total(uint32_t* scratch);
 void launch_scan(const Launch& L, const uint2* counts, int64_t n, uint32_t* inst_off, uint64_t* pair_off,
-                 ulonglong2* parts, int64_t n_parts_cap);
+                 uint32_t* scratch, uint32_t* err, uint64_t spin_ns);
 
 // K2: for every visible instance of views [v0, v1): its record, identity, depth key
 // (bits(z32) - zbase saturated to 28 bits), its own index (the value the depth sort carries)

@@ -123,8 +123,7 @@ extern "C" int dgs_render_noalloc(const dgs_options* opt, const dgs_node* nodes,
     uint2* d_counts = cv.take<uint2>(T);
     uint32_t* d_inst_off = cv.take<uint32_t>(T + 1);
     uint64_t* d_pair_off = cv.take<uint64_t>(T + 1);
-    const int64_t n_parts = (T + 4095) / 4096;
-    ulonglong2* d_parts = cv.take<ulonglong2>(n_parts + 1);
+    uint32_t* d_scan = cv.take<uint32_t>(scan_words(T));
     uint64_t* d_rb = cv.take<uint64_t>(2 * (V + 1) + 1);
     if (!cv.ok) return DGS_ERR_CAPACITY;
 
@@ -146,12 +145,13 @@ extern "C" int dgs_render_noalloc(const dgs_options* opt, const dgs_node* nodes,
     launch_setup_views(L, d_views, V, node_poses, d_slot, K, d_vnodes, d_vtab, d_err);
     launch_count(L, dtype_mask, d_nodes, n_nodes, d_views, d_vnodes, K, d_nv, d_nvoff, (int)chunk_total, P, 0, V, true,
                  nullptr, 0, d_counts);
-    launch_scan(L, d_counts, T, d_inst_off, d_pair_off, d_parts, n_parts + 1);
+    NA_CUDA(cudaMemsetAsync(d_scan, 0, sizeof(uint32_t) * scan_words(T), stream));
+    launch_scan(L, d_counts, T, d_inst_off, d_pair_off, d_scan, d_err, SortCtl{}.spin_ns);
     // one view group: read back the grand totals and the error word
     NA_CUDA(cudaMemsetAsync(d_rb, 0, sizeof(uint64_t) * 3, stream));
     // the 64-bit instance total of the scan (its 32-bit offsets wrap beyond 2^32)
-    if (n_parts > 0)
-        NA_CUDA(cudaMemcpyAsync(d_rb, d_parts + n_parts, sizeof(uint64_t), cudaMemcpyDeviceToDevice, stream));
+    if (T > 0)
+        NA_CUDA(cudaMemcpyAsync(d_rb, scan_total(d_scan), sizeof(uint64_t), cudaMemcpyDeviceToDevice, stream));
     NA_CUDA(cudaMemcpyAsync(d_rb + 1, d_pair_off + T, sizeof(uint64_t), cudaMemcpyDeviceToDevice, stream));
     NA_CUDA(cudaMemcpyAsync(d_rb + 2, d_err, sizeof(uint32_t), cudaMemcpyDeviceToDevice, stream));
     uint64_t h_rb[3] = {0, 0, 0};
@@ -160,6 +160,7 @@ extern "C" int dgs_render_noalloc(const dgs_options* opt, const dgs_node* nodes,
     NA_CUDA(cudaStreamSynchronize(stream));
     const uint64_t n_vis = h_rb[0], n_pairs = h_rb[1];
     if ((uint32_t)h_rb[2] & kErrPose) return DGS_ERR_INVALID_ARG;
+    if ((uint32_t)h_rb[2] & kErrTimeout) return DGS_ERR_TIMEOUT;
     if (n_pairs > kMaxPairs || n_vis >= (1ull << 32)) return DGS_ERR_CAPACITY;
 
     // ---------------------------------------------------------------- phase 2 scratch

@@ -804,8 +804,7 @@ __device__ __forceinline__ void block_excl_scan2(uint64_t& a, uint64_t& b, uint6
 // both access patterns free of bank conflicts.
 constexpr int kScanPadded = kScanTile + kScanTile / 16;
 __device__ __forceinline__ int scan_slot(int k) { return k + (k >> 4); }
-__device__ __forceinline__ void load_tile_counts(const uint2* __restrict__ counts, int64_t n, uint2* s_c) {
-    const int64_t b0 = (int64_t)blockIdx.x * kScanTile;
+__device__ __forceinline__ void load_tile_counts(const uint2* __restrict__ counts, int64_t b0, int64_t n, uint2* s_c) {
 #pragma unroll 4
     for (int j = 0; j < kScanItems; ++j) {
         const int k = j * kScanThreads + threadIdx.x;
@@ -814,43 +813,65 @@ __device__ __forceinline__ void load_tile_counts(const uint2* __restrict__ count
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_partial(const uint2* __restrict__ counts, int64_t n, ulonglong2* parts) {
-    __shared__ uint2 s_c[kScanPadded];
-    load_tile_counts(counts, n, s_c);
-    uint64_t a = 0, b = 0;
-    for (int j = 0; j < kScanItems; ++j) {
-        const uint2 c = s_c[scan_slot(threadIdx.x * kScanItems + j)];
-        a += __popc(c.x); b += c.y;
+// Decoupled look-back over 64-bit sums (a 2-bit flag above 62 bits), by one warp: publishes this
+// partition's sum and returns the sum of those before it.  Bounded like the sort's.
+constexpr uint64_t kAgg64 = 1ull << 62, kInc64 = 2ull << 62, kSum64 = (1ull << 62) - 1ull;
+
+__device__ __forceinline__ uint64_t look_back64(uint64_t* status, int64_t part, uint64_t sum, int lane, uint32_t* err,
+                                                uint64_t spin_ns) {
+    auto ld = [&](int64_t i) {
+        uint64_t v;
+        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(status + i) : "memory");
+        return v;
+    };
+    auto st = [&](uint64_t v) { asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(status + part), "l"(v) : "memory"); };
+    if (lane == 0) st((part == 0 ? kInc64 : kAgg64) | sum);
+    if (part == 0) return 0;
+    uint64_t excl = 0, t0 = 0;
+    uint32_t spins = 0;
+    for (int64_t p = part - 1;;) {
+        const uint64_t sv = p - lane >= 0 ? ld(p - lane) : kInc64;
+        const uint64_t f = sv & ~kSum64;
+        const uint32_t inc = __ballot_sync(0xffffffffu, f == kInc64), none = __ballot_sync(0xffffffffu, f == 0);
+        const int last = inc ? __ffs(inc) - 1 : 31;         // the predecessors up to here are summed
+        if ((none & ((2u << last) - 1u)) == 0) {
+            uint64_t x = lane <= last ? sv & kSum64 : 0ull;
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            excl += x;
+            if (inc) break;
+            p -= 32;
+            continue;
+        }
+        bool expired = false;
+        if ((++spins & 255u) == 0) {
+            const uint64_t now = global_timer_ns();
+            if (t0 == 0) t0 = now;
+            else expired = now - t0 > spin_ns;
+        }
+        if (__any_sync(0xffffffffu, expired)) {
+            if (lane == 0) atomicOr(err, kErrTimeout);
+            break;
+        }
     }
-    uint64_t ta, tb;
-    block_excl_scan2(a, b, ta, tb);
-    if (threadIdx.x == 0) parts[blockIdx.x] = make_ulonglong2(ta, tb);
+    if (lane == 0) st(kInc64 | ((excl + sum) & kSum64));
+    return excl;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_parts(ulonglong2* parts, int64_t n_parts) {
-    // single block: exclusive scan of the per-tile totals, in place; parts[n_parts] = grand total
-    __shared__ uint64_t carry_a, carry_b;
-    if (threadIdx.x == 0) { carry_a = 0; carry_b = 0; }
+// Exclusive scan of the count table's instances and pair bounds in one pass: a block takes the next
+// kScanTile entries from a counter, and warps 0 and 1 find the sums before them.  Entry n and *total
+// receive the totals.  After a wait that ran out (kErrTimeout) the offsets are not valid: the host,
+// or the graph's size check, stops the call before anything is written through them.
+__global__ void __launch_bounds__(kScanThreads) k_scan(const uint2* __restrict__ counts, int64_t n, uint32_t* counter,
+                                                      uint64_t* status, ulonglong2* total, uint32_t* inst_off,
+                                                      uint64_t* pair_off, uint32_t* err, uint64_t spin_ns) {
+    __shared__ uint2 s_c[kScanPadded];
+    __shared__ uint32_t s_part;
+    __shared__ uint64_t s_excl[2];
+    if (threadIdx.x == 0) s_part = atomicAdd(counter, 1u);
     __syncthreads();
-    for (int64_t base = 0; base < n_parts; base += kScanThreads) {
-        const int64_t i = base + threadIdx.x;
-        uint64_t a = 0, b = 0;
-        if (i < n_parts) { a = parts[i].x; b = parts[i].y; }
-        uint64_t ta, tb;
-        block_excl_scan2(a, b, ta, tb);
-        if (i < n_parts) parts[i] = make_ulonglong2(a + carry_a, b + carry_b);
-        __syncthreads();
-        if (threadIdx.x == 0) { carry_a += ta; carry_b += tb; }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) parts[n_parts] = make_ulonglong2(carry_a, carry_b);
-}
-
-__global__ void __launch_bounds__(kScanThreads) k_scan_final(const uint2* __restrict__ counts, int64_t n,
-                                                            const ulonglong2* __restrict__ parts, uint32_t* inst_off,
-                                                            uint64_t* pair_off) {
-    __shared__ uint2 s_c[kScanPadded];
-    load_tile_counts(counts, n, s_c);
+    const int64_t part = s_part, parts = gridDim.x, b0 = part * kScanTile;
+    load_tile_counts(counts, b0, n, s_c);
     uint2 c[kScanItems];
     uint64_t a = 0, b = 0;
     for (int j = 0; j < kScanItems; ++j) {
@@ -859,16 +880,20 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_final(const uint2* __rest
     }
     uint64_t ta, tb;
     block_excl_scan2(a, b, ta, tb);
-    a += parts[blockIdx.x].x;
-    b += parts[blockIdx.x].y;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp < 2) {
+        const uint64_t e = look_back64(status + warp * parts, part, warp ? tb : ta, lane, err, spin_ns);
+        if (lane == 0) s_excl[warp] = e;
+    }
+    __syncthreads();
+    a += s_excl[0];
+    b += s_excl[1];
     // the offsets go back through shared memory so that the stores are warp-striped too; entry
     // n, inside the tile or just past the last one, receives the totals
-    const int64_t b0 = (int64_t)blockIdx.x * kScanTile;
     uint64_t* s_p = reinterpret_cast<uint64_t*>(s_c);
     uint32_t* s_i = reinterpret_cast<uint32_t*>(s_c);
     const uint64_t a0 = a;
-    __syncthreads();                            // every thread has read its counts
-    for (int j = 0; j < kScanItems; ++j) {
+    for (int j = 0; j < kScanItems; ++j) {      // (every thread has read its counts: the barrier above)
         s_p[scan_slot(threadIdx.x * kScanItems + j)] = b;
         b += c[j].y;
     }
@@ -890,8 +915,9 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_final(const uint2* __rest
         const int k = j * kScanThreads + threadIdx.x;
         if (b0 + k <= n) inst_off[b0 + k] = s_i[scan_slot(k)];
     }
-    if (n % kScanTile == 0 && blockIdx.x == gridDim.x - 1 && threadIdx.x == kScanThreads - 1) {
-        inst_off[n] = (uint32_t)a; pair_off[n] = b;
+    if (part == parts - 1 && threadIdx.x == kScanThreads - 1) {
+        if (n % kScanTile == 0) { inst_off[n] = (uint32_t)a; pair_off[n] = b; }
+        *total = make_ulonglong2(a, b);
     }
 }
 
@@ -973,19 +999,21 @@ void launch_emit(const Launch& L, int dtype_mask, const NodeDesc* nodes, int n_n
                              batched, pmap, view_chunks, counts, inst_off, inst_base, out);
 }
 
+size_t scan_words(int64_t n) { return 8 + 4 * (size_t)((n + kScanTile - 1) / kScanTile); }
+
+ulonglong2* scan_total(uint32_t* scratch) { return reinterpret_cast<ulonglong2*>(scratch + 4); }
+
 void launch_scan(const Launch& L, const uint2* counts, int64_t n, uint32_t* inst_off, uint64_t* pair_off,
-                 ulonglong2* parts, int64_t n_parts_cap) {
+                 uint32_t* scratch, uint32_t* err, uint64_t spin_ns) {
     const int64_t n_parts = (n + kScanTile - 1) / kScanTile;
-    (void)n_parts_cap;
     if (n_parts == 0) {
         cudaMemsetAsync(inst_off, 0, sizeof(uint32_t), L.stream);
         cudaMemsetAsync(pair_off, 0, sizeof(uint64_t), L.stream);
         return;
     }
-    k_scan_partial<<<(unsigned)n_parts, kScanThreads, 0, L.stream>>>(counts, n, parts);
-    k_scan_parts<<<1, kScanThreads, 0, L.stream>>>(parts, n_parts);
-    k_scan_final<<<(unsigned)n_parts, kScanThreads, 0, L.stream>>>(counts, n, parts, inst_off, pair_off);
-    *L.launches += 3;
+    k_scan<<<(unsigned)n_parts, kScanThreads, 0, L.stream>>>(counts, n, scratch, reinterpret_cast<uint64_t*>(scratch + 8),
+                                                             scan_total(scratch), inst_off, pair_off, err, spin_ns);
+    ++*L.launches;
 }
 
 }  // namespace dgs
