@@ -67,7 +67,8 @@ __device__ __forceinline__ float warp_transpose_sum16(const float (&v)[16], int 
 // Measured against reducing every pair's ten partials over the warp by shuffles (16 per record,
 // about 190 instructions in all, 10 scalar atomics): one 800x800 view with 241k instances
 // 0.216 -> 0.136 ms, four 401x301 views without checkpoints (one warp per whole list: the longest
-// lists are the time) 0.360 -> 0.231.
+// lists are the time) 0.360 -> 0.231; and with the gradients of kStep records side by side in place
+// of one divergent branch per record 0.127 and 0.204.  kStep 8 is slower on the first, 2 on the second.
 constexpr int kHalf = 16;                       // records per replay
 constexpr int kScan = 4;                        // list entries per lane and scan step
 constexpr int kQueue = 256;                     // ring of queued entries: at most 31 + 32 kScan are held
@@ -90,7 +91,7 @@ __device__ __forceinline__ void red_add2(float* p, float a, float b) {
     asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(a), "f"(b) : "memory");
 }
 
-__global__ void __launch_bounds__(kCompWarps * 32) k_composite_bwd(const ViewDesc* __restrict__ views, int v0, int nv,
+__global__ void __launch_bounds__(kCompWarps * 32, 10) k_composite_bwd(const ViewDesc* __restrict__ views, int v0, int nv,
                                                        const uint2* __restrict__ ranges, const uint32_t* __restrict__ keys,
                                                        const uint32_t* __restrict__ vals,
                                                        const Record* __restrict__ rec, Params P,
@@ -243,26 +244,39 @@ __global__ void __launch_bounds__(kCompWarps * 32) k_composite_bwd(const ViewDes
                     raw[u] = r1.z * ex[u];
                     al[u] = hit[u] ? fminf(P.alpha_max, raw[u]) : 0.f;
                 }
+                // the transmittance through the records in order, then the gradients of all of them
+                // (independent of each other; a branch per record would put them one behind the other)
+                float Tb[kStep], Ta[kStep];
+                float2 Q01[kStep], Q2d[kStep];
+                bool con[kStep];
 #pragma unroll
                 for (int u = 0; u < kStep; ++u) {
                     const float4 r2 = S.rec[2][k0 + k + u];
                     const float Tn = fmaf(-al[u], T, T);      // T (1 - alpha), one rounding
                     const bool go = __float_as_int(Tn) >= tmin;
-                    float2 we = make_float2(0.f, 0.f);
-                    if (go && hit[u]) {
-                        we.x = al[u] * T;
-                        const float2 c01 = make_float2(r2.x, r2.y), c2d = make_float2(r2.z, r2.w), w2 = make_float2(we.x, we.x);
-                        P01 = fma2(w2, c01, P01);
-                        P2d = fma2(w2, c2d, P2d);
-                        const float iTn = __fdividef(1.f, Tn);   // Tn >= t_min > 0
-                        const float S0 = (Co01.x - P01.x) * iTn, S1 = (Co01.y - P01.y) * iTn;
-                        const float S2 = (Co2d.x - P2d.x) * iTn, SD = (Co2d.y - P2d.y) * iTn;
-                        const float dal = T * (g01.x * (c01.x - S0) + g01.y * (c01.y - S1) + g2d.x * (c2d.x - S2) +
-                                               g2d.y * (c2d.y - SD));
-                        we.y = raw[u] > P.alpha_max ? 0.f : dal * ex[u];
+                    con[u] = go && hit[u];
+                    Tb[u] = T;
+                    Ta[u] = Tn;
+                    const float wgt = al[u] * T;
+                    if (con[u]) {
+                        const float2 w2 = make_float2(wgt, wgt);
+                        P01 = fma2(w2, make_float2(r2.x, r2.y), P01);
+                        P2d = fma2(w2, make_float2(r2.z, r2.w), P2d);
                     }
+                    Q01[u] = P01;
+                    Q2d[u] = P2d;
                     T = go ? Tn : __int_as_float(__float_as_int(T) | 0x80000000);   // (-|T|)
-                    S.we[k + u][lane] = we;
+                }
+#pragma unroll
+                for (int u = 0; u < kStep; ++u) {
+                    const float4 r2 = S.rec[2][k0 + k + u];
+                    const float iTn = __fdividef(1.f, Ta[u]);   // Tn >= t_min > 0 where it counts
+                    const float S0 = (Co01.x - Q01[u].x) * iTn, S1 = (Co01.y - Q01[u].y) * iTn;
+                    const float S2 = (Co2d.x - Q2d[u].x) * iTn, SD = (Co2d.y - Q2d[u].y) * iTn;
+                    const float dal = Tb[u] * (g01.x * (r2.x - S0) + g01.y * (r2.y - S1) + g2d.x * (r2.z - S2) +
+                                               g2d.y * (r2.w - SD));
+                    S.we[k + u][lane] = make_float2(con[u] ? al[u] * Tb[u] : 0.f,
+                                                    con[u] && !(raw[u] > P.alpha_max) ? dal * ex[u] : 0.f);
                 }
                 if (__all_sync(0xffffffffu, T < 0.f)) { ended = true; kn = k + kStep; break; }
             }
