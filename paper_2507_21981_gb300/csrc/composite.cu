@@ -445,7 +445,7 @@ void launch_composite(const Launch& L, const ViewDesc* views, int v0, int n_grou
     if (n_tiles == 0) return;
     // checkpoints are for the adjoint, which never runs on randomised outputs
     const bool with_ck = ck.st != nullptr && !P.aug;
-    // few waves: fewer resident blocks with more registers (no spills) shorten the longest lists' chains;
+    // few waves: fewer resident blocks with more registers shorten the longest lists' chains;
     // many waves: the most blocks that fit.  One-group times with 14 against 16 blocks an SM: 64 tiles
     // 16.4 against 18.4 us, 2400 tiles 71.6 / 80, 19200 tiles 268 / 264, 153600 tiles 3986 / 3907.
     const bool few = n_tiles <= 4096;
