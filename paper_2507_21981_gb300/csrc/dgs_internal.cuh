@@ -690,7 +690,7 @@ struct TsdfParams {
 };
 // host_views: the V views; up to kTsdfParamViews of them travel as a kernel parameter, more are
 // read from table (the same views in device memory).  dn: scratch of one float per pixel.
-constexpr int kTsdfParamViews = 40;
+constexpr int kTsdfParamViews = 128;     // 12 KB of kernel parameters
 struct TsdfViews {
     TsdfView v[kTsdfParamViews];
 };

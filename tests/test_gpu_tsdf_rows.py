@@ -1,7 +1,7 @@
 """The fusion kernels' split over row lengths (dgs_tsdf_integrate) against the FP64 oracle: rows
 below, at and above one round of 32 voxels, one, two and four rounds per warp with remainders, both
 forms of the voxel centre (row length a multiple of four or not), and view tables passed with the
-launch (up to 40 views) or read from memory.  Tolerances are those of test_gpu_tsdf.py: the weight
+launch (up to 128 views) or read from memory.  Tolerances are those of test_gpu_tsdf.py: the weight
 exactly and the field within 1e-4, away from the decisions the oracle flags."""
 import numpy as np
 import pytest
@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("nx,n_views", [(7, 5), (28, 5), (31, 5), (32, 40), (33, 41), (61, 5), (64, 5), (100, 5),
-                                        (130, 5), (200, 5), (257, 5)])
+                                        (130, 5), (200, 5), (257, 5), (40, 128), (45, 129), (20, 129)])
 def test_rows(nx, n_views):
     c = np.array([0.05, -0.1, 0.1])
     cams, Dv, Av = S.sphere_depth_views(c, 0.2, n_views=n_views, width=72, height=56, f=64.0, dist=1.0, seed=nx)
