@@ -47,9 +47,9 @@ PROJ_OPS, SH3_OPS, CULL_OPS = 200, 90, 35
 # read, 236 B of attribute gradients accumulated and 8 B of identity.
 PROJECT_BWD_BYTES = 40 + 236 + 236 + 8
 # DRAM bytes (read + write) per launch on the full workload, from a one-pass ncu capture
-# (dram__bytes_read.sum + dram__bytes_write.sum) of the full launch: 1005.0 + 754.6 MB.  Set to
+# (dram__bytes_read.sum + dram__bytes_write.sum) of the full launch: 1043.7 + 756.3 MB.  Set to
 # None whenever the kernel changes after its capture.
-TRAFFIC = {"composite": 1.7596e9}
+TRAFFIC = {"composite": 1.8000e9}
 # FP32 operations per (voxel, view) of the TSDF fusion: camera-space point (9 FMA), reciprocal,
 # projection (4), bounds (4 compares), coverage test, normalised depth (2), sdf, truncation,
 # clamp (2), running average (3), weight update (2)
@@ -885,20 +885,20 @@ def main():
     dom = max(per_step, key=per_step.get)
     P, NV = stats["n_pairs"], stats["n_visible"]
     passes = (stats["key_bits"] + 7) // 8          # tile-sort passes (key_bits = tile key bits)
-    # passes of the depth sort's view key (the bits of the views per group; none for one view);
-    # the view rides in the instance numbers' high bits when both fit in 32 bits, else each
-    # view pass also gathers the view of every value (4 B)
+    # passes of the depth sort's view key (the bits of the views per group; none where up to 16
+    # views lie above the depth key in its 32 bits); the view rides in the instance numbers' high
+    # bits when both fit in 32 bits, else each view pass also gathers the view of every value (4 B)
     vpg = -(-stats["n_views"] // max(stats["n_groups"], 1))
     vbits = (vpg - 1).bit_length()
-    vpasses = (vbits + 7) // 8
+    vpasses = (vbits + 7) // 8 if vbits > 4 else 0
     packed = vbits > 0 and (max(NV // max(stats["n_groups"], 1), 1) - 1).bit_length() + vbits <= 32
     # algorithmic bytes of the binning class: depth sort of the instances (28-bit keys: the
     # histogram read, 4 passes of 16 B, the last writing no keys when view passes follow; each
-    # view pass reads and writes the value), tile-count scan (order and count read twice, offset
-    # written: 20 B), pair emission (record 48 + identity 8 + order 4 + offset 4 read; 8 B
+    # view pass reads and writes the value), tile-count scan (order and count read, offset
+    # written: 12 B), pair emission (record 48 + identity 8 + order 4 + offset 4 read; 8 B
     # written per pair) and the tile sort (histogram read, passes of 16 B)
     depth_b = 4 + 4 * 16 - (4 if vpasses else 0) + vpasses * (8 if packed else 12)
-    sort_bytes = NV * (depth_b + 20 + 64) + P * (8 + 4 + passes * 16)
+    sort_bytes = NV * (depth_b + 12 + 64) + P * (8 + 4 + passes * 16)
     # compositor work of one step, counted by the instrumented compositor outside the timed region
     rc_ = Renderer(mode="batched", tile=tile, profile=2)
     rc_.render(ds, out=out)
@@ -924,7 +924,7 @@ def main():
         "sort": {**hbm(sort_bytes, per_step["sort"]),
                  "units": {"instances": NV, "pairs": P, "depth_passes": 4, "view_passes": vpasses,
                            "view_key": "packed in the values" if packed else "gathered",
-                           "tile_passes": passes, "bytes_per_instance": depth_b + 20 + 64,
+                           "tile_passes": passes, "bytes_per_instance": depth_b + 12 + 64,
                            "bytes_per_pair": 8 + 4 + passes * 16}},
         "emit": {**alu(NV * (PROJ_OPS + SH3_OPS), per_step["emit"]),
                  "units": {"visible": NV, "ops_per_visible": PROJ_OPS + SH3_OPS,
