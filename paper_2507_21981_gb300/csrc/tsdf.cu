@@ -208,7 +208,9 @@ static void tsdf_launch(const Launch& L, float* F, float* W, int nx, int ny, int
         k_tsdf<BY_VALUE><<<(unsigned)((n_vox + kTsdfThreads - 1) / kTsdfThreads), kTsdfThreads, 0, L.stream>>>(
             F, W, nx, ny, n_vox, TP, set, table, V, dn);
     } else {
-        // the widest segment that leaves at most a fifth more lanes idle than single rounds do
+        // the widest segment that leaves at most a fifth more lanes idle than single rounds do (128 x 128
+        // rows, 16 views, against the four-voxel kernel: rows of 33 voxels 59 -> 50 us, 36 53 -> 49, 50 74 ->
+        // 49, 98 114 -> 72, 130 141 -> 102, 250 232 -> 117; of 24, by k_tsdf, 49 -> 39)
         const int rounds = (nx + 31) / 32;
         const int NR = (rounds + 3) / 4 * 4 * 5 <= rounds * 6 ? 4 : (rounds + 1) / 2 * 2 * 5 <= rounds * 6 ? 2 : 1;
         const int segs = (rounds + NR - 1) / NR;
