@@ -313,10 +313,12 @@ __device__ __forceinline__ uint64_t cut_pending(RayWarp& W, int& cnt, int lane) 
 // hits beyond them are skipped, and another round resumes after them.  The trees of up to 32
 // slots share one stack; with more, a slot batch is traversed after the other and hits are
 // final at the end of the round only.
-// Bound by latency (boxes and records come from L2, one dependent load per step), which the 24
-// or more warps per SM hide.  Measured against a packet of 32 rays per warp with a 32-hit buffer
-// per lane, same outputs bit for bit: one sensor of 32 x 1024 beams through 380k Gaussians 0.53 ms
-// against 7.4 (there the slowest packet was the time), 16 sensors through 580k 6.0 ms against 28.
+// Bound by latency (boxes and records come from L2, one dependent load per step) and at 66 % issue;
+// 64 registers keep 32 warps an SM.  Same outputs bit for bit, one sensor of 32 x 1024 beams through
+// 380k Gaussians and 16 sensors through 580k: a packet of 32 rays per warp with a 32-hit buffer per
+// lane 7.4 and 28 ms (with one sensor the slowest packet was the time); one ray per warp, one node
+// of five levels per expansion, 72 registers 0.592 and 5.59 ms; two nodes 0.588 and 5.51; with 64
+// registers 0.555 and 5.04.
 __global__ void __launch_bounds__(kRayWarps * 32, 8) k_lidar_trace(const LidarTreeDev* __restrict__ trees,
                                                                 const LidarSlot* __restrict__ slots, int K,
                                                                 const float* __restrict__ dirs, int n_dirs,
