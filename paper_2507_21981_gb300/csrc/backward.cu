@@ -77,7 +77,7 @@ static_assert(kQueue >= 31 + 32 * kScan && (kQueue & (kQueue - 1)) == 0, "ring s
 
 struct BwdWarp {
     float4 rec[3][32];                          // (-u, -v, c qa, c qc), (qb, threshold, o, qa), (r, g, b, z)
-    float4 pix[32];                             // the pixels' upstream gradients
+    float4 pix[32];                             // the pixels' upstream gradients (zero where not finite)
     float2 we[kHalf][33];                       // [record][pixel] (w, e)
     float qc[32];
     uint32_t idx[32];
@@ -144,6 +144,10 @@ __global__ void __launch_bounds__(kCompWarps * 32, 10) k_composite_bwd(const Vie
         Co2d = make_float2(out_rgb[p * 3 + 2], out_depth[p]);
     }
     if (__all_sync(0xffffffffu, g01.x == 0.f && g01.y == 0.f && g2d.x == 0.f && g2d.y == 0.f)) return;
+    // pixels whose upstream gradient is NaN or infinite (0 times infinity of a masked division, say, at
+    // a pixel that nothing covers): they take part only in the records that reach them
+    const bool fin = isfinite(g01.x) && isfinite(g01.y) && isfinite(g2d.x) && isfinite(g2d.y);
+    const uint32_t odd = __ballot_sync(0xffffffffu, !fin);
     uint2 range = ranges[gt];
     uint32_t reds = 0;
     float T = inside ? 1.f : -1.f;              // < 0 marks a pixel that has ended, as in the forward
@@ -166,7 +170,7 @@ __global__ void __launch_bounds__(kCompWarps * 32, 10) k_composite_bwd(const Vie
     const uint32_t lt = (1u << lane) - 1u;
     const uint32_t wbit = 1u << (kTileBits + w);
     BwdWarp& S = s_warp[bw];
-    S.pix[lane] = make_float4(g01.x, g01.y, g2d.x, g2d.y);
+    S.pix[lane] = fin ? make_float4(g01.x, g01.y, g2d.x, g2d.y) : make_float4(0.f, 0.f, 0.f, 0.f);
     const int row = lane & (kHalf - 1), half = lane >> 4;      // the sum's record and pixel rows 2 half, 2 half + 1
 
     // the list's selected entries, queued as the forward queues them
@@ -315,6 +319,15 @@ __global__ void __launch_bounds__(kCompWarps * 32, 10) k_composite_bwd(const Vie
                 syy = fmaf(dy * dy, e1, syy);
             }
             const uint32_t full = 0xffffffffu;
+            // (staged as zeros, and a zero weight leaves them out: 0 times NaN would not)
+            for (uint32_t rest = odd; rest; rest &= rest - 1) {
+                const int p = __ffs(rest) - 1;
+                const float4 g = make_float4(__shfl_sync(full, g01.x, p), __shfl_sync(full, g01.y, p),
+                                             __shfl_sync(full, g2d.x, p), __shfl_sync(full, g2d.y, p));
+                const float we = S.we[row][p].x;
+                if ((p >> 4) == half && we != 0.f)
+                    sg = make_float4(fmaf(we, g.x, sg.x), fmaf(we, g.y, sg.y), fmaf(we, g.z, sg.z), fmaf(we, g.w, sg.w));
+            }
             any |= __shfl_xor_sync(full, any, kHalf);
             s1 += __shfl_xor_sync(full, s1, kHalf);
             st += __shfl_xor_sync(full, st, kHalf);
