@@ -393,6 +393,10 @@ class DGSRenderFn(torch.autograd.Function):
     def forward(ctx, renderer, ds, node_poses, *params):
         ds.set_poses(node_poses.detach())
         rgb, depth, alpha = renderer.render(ds)
+        if renderer.mode == "graph":
+            # the renderer's own tensors, which its next render overwrites unseen by autograd: a node
+            # saves and returns copies
+            rgb, depth, alpha = rgb.clone(), depth.clone(), alpha.clone()
         ctx.renderer, ctx.ds = renderer, ds
         ctx.save_for_backward(rgb, depth)
         ctx.pose_shape = node_poses.shape
