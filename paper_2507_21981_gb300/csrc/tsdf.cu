@@ -17,6 +17,7 @@ namespace dgs {
 namespace {
 
 constexpr int kTsdfThreads = 256;
+constexpr int kLaneVox = 4;          // voxels per lane of the fusion kernels
 
 // The view table: by value as a kernel parameter for up to kTsdfParamViews views, whose fields are
 // then constant-bank operands (from shared memory their broadcasts were half of the data path),
@@ -72,7 +73,7 @@ __device__ __forceinline__ void voxel_x(int i, int nx, const TsdfParams& TP, flo
 }
 
 // Non-negative floats order like their bit patterns, negative ones and NaN lie above them: one
-// integer comparison for 0 <= u < W (u is never -0: cx and cy are not).
+// integer comparison for 0 <= u < W (u = -0 is a product that underflowed below zero: cx and cy are not -0).
 __device__ __forceinline__ bool in_range(float u, float W) { return __float_as_uint(u) < __float_as_uint(W); }
 
 // 1 / x for normal x: the approximate division below without its range handling (a pixel's z and
@@ -102,49 +103,78 @@ __device__ __forceinline__ void fuse(float d, float z, bool ok, const TsdfParams
     w = fminf(w + 1.f, TP.max_weight);
 }
 
-// Rows of fewer than 32 voxels: one thread per voxel in storage order.
+// Warp = 32 kLaneVox consecutive voxels in storage order, lane + 32 m the m-th of a lane, whatever rows
+// they belong to: for rows that k_tsdf_rows would pad with idle lanes.  The view's fields are read once
+// for a lane's voxels, as there; nothing is shared along a row.  256 x 256 rows, 32 views of 640x480,
+// a voxel of 1.2 px, with the pre-pass, against four adjacent voxels per thread with the view table in
+// shared memory (one per thread where the row length is no multiple of four), and against segments
+// of one row with one or two voxels per lane: rows of 28 voxels 190 / 199 -> 126 us, 33 248 / 235 -> 142, 64
+// 330 / 240 -> 236, 80 396 / 406 -> 285, 129 751 / 635 -> 442.
 template <bool BY_VALUE>
 __global__ void __launch_bounds__(kTsdfThreads) k_tsdf(float* __restrict__ F, float* __restrict__ Wt, int nx, int ny,
                                                        int64_t n_vox, TsdfParams TP,
                                                        const __grid_constant__ TsdfViews set,
                                                        const TsdfView* __restrict__ table, int V,
                                                        const float* __restrict__ dn) {
-    const int64_t idx = (int64_t)blockIdx.x * kTsdfThreads + threadIdx.x;
-    if (idx >= n_vox) return;
-    const int i = (int)(idx % nx);
-    const int64_t r = idx / nx;
-    const int j = (int)(r % ny), k = (int)(r / ny);
-    float px, m;
-    voxel_x(i, nx, TP, px, m);
-    const float py = fmaf((float)j + 0.5f, TP.voxel, TP.oy), pz = fmaf((float)k + 0.5f, TP.voxel, TP.oz);
-    float f = F[idx], w = Wt[idx];
+    // (fewer than 2^31 voxels: 32-bit indices)
+    const uint32_t idx0 = (blockIdx.x * (kTsdfThreads / 32u) + (threadIdx.x >> 5)) * (32u * kLaneVox) + lane_id();
+    const uint32_t n = (uint32_t)n_vox;
+    float px[kLaneVox], py[kLaneVox], pz[kLaneVox], ms[kLaneVox], f[kLaneVox], w[kLaneVox];
+#pragma unroll
+    for (int m = 0; m < kLaneVox; ++m) {
+        const uint32_t idx = idx0 + 32u * m, r = idx / (uint32_t)nx, k = r / (uint32_t)ny;
+        voxel_x((int)(idx - r * (uint32_t)nx), nx, TP, px[m], ms[m]);
+        if (idx >= n) px[m] = __int_as_float(0x7fc00000);   // no view sees it
+        py[m] = fmaf((float)(int)(r - k * (uint32_t)ny) + 0.5f, TP.voxel, TP.oy);
+        pz[m] = fmaf((float)(int)k + 0.5f, TP.voxel, TP.oz);
+        f[m] = idx < n ? F[idx] : 0.f;
+        w[m] = idx < n ? Wt[idx] : 0.f;
+    }
     for (int v = 0; v < V; ++v) {
         const TsdfView& cv = view_of<BY_VALUE>(set, table, v);
-        const float z0 = fmaf(cv.R[6], px, fmaf(cv.R[7], py, fmaf(cv.R[8], pz, cv.t[2])));
-        const float x0 = fmaf(cv.R[0], px, fmaf(cv.R[1], py, fmaf(cv.R[2], pz, cv.t[0])));
-        const float y0 = fmaf(cv.R[3], px, fmaf(cv.R[4], py, fmaf(cv.R[5], pz, cv.t[1])));
-        const float z = fmaf(m, cv.R[6] * TP.voxel, z0);
-        const float x = fmaf(m, cv.R[0] * TP.voxel, x0), y = fmaf(m, cv.R[3] * TP.voxel, y0);
-        const float iz = rcp(z);
-        const float u = fmaf(cv.fx * x, iz, cv.cx), vv = fmaf(cv.fy * y, iz, cv.cy);
-        const bool ok = z > 0.f && in_range(u, cv.Wf) && in_range(vv, cv.Hf);
-        const float d = ok ? __ldg(dn + cv.q0 + pixel_of(u, vv, (uint32_t)cv.W)) : 0.f;
-        fuse(d, z, ok, TP, f, w);
+        const float sx = cv.R[0] * TP.voxel, sy = cv.R[3] * TP.voxel, sz = cv.R[6] * TP.voxel;
+        const float cx = cv.cx, cy = cv.cy, Wf = cv.Wf, Hf = cv.Hf;
+        const uint32_t W = (uint32_t)cv.W;
+        const float* __restrict__ dv = dn + cv.q0;
+        float zm[kLaneVox], d[kLaneVox];
+        uint32_t pix[kLaneVox];
+        bool ok[kLaneVox];
+#pragma unroll
+        for (int m = 0; m < kLaneVox; ++m) {
+            const float z0 = fmaf(cv.R[6], px[m], fmaf(cv.R[7], py[m], fmaf(cv.R[8], pz[m], cv.t[2])));
+            const float x0 = fmaf(cv.R[0], px[m], fmaf(cv.R[1], py[m], fmaf(cv.R[2], pz[m], cv.t[0])));
+            const float y0 = fmaf(cv.R[3], px[m], fmaf(cv.R[4], py[m], fmaf(cv.R[5], pz[m], cv.t[1])));
+            const float z = fmaf(ms[m], sz, z0);
+            const float x = fmaf(ms[m], sx, x0), y = fmaf(ms[m], sy, y0);
+            const float iz = rcp(z);
+            const float u = fmaf(cv.fx * x, iz, cx), vv = fmaf(cv.fy * y, iz, cy);
+            ok[m] = z > 0.f && in_range(u, Wf) && in_range(vv, Hf);
+            pix[m] = pixel_of(u, vv, W);                // (below 2^30 where it is used)
+            zm[m] = z;
+        }
+#pragma unroll
+        for (int m = 0; m < kLaneVox; ++m) d[m] = ok[m] ? __ldg(dv + pix[m]) : 0.f;
+#pragma unroll
+        for (int m = 0; m < kLaneVox; ++m) fuse(d[m], zm[m], ok[m], TP, f[m], w[m]);
     }
-    F[idx] = f;
-    Wt[idx] = w;
+#pragma unroll
+    for (int m = 0; m < kLaneVox; ++m) {
+        const uint32_t idx = idx0 + 32u * m;
+        if (idx < n) {
+            F[idx] = f[m];
+            Wt[idx] = w[m];
+        }
+    }
 }
 
-// Warp = NR x 32 consecutive voxels of one row, lane + 32 m the m-th of a lane: neighbouring lanes
+// Warp = kLaneVox x 32 consecutive voxels of one row, lane + 32 m the m-th of a lane: neighbouring lanes
 // hold neighbouring voxels, whose projections share the 32-byte sectors of the depth image, the
-// NR projections are made before the NR gathers, which are then in flight together, and the
+// kLaneVox projections are made before the gathers, which are then in flight together, and the
 // row's part of the camera transform is shared.  Each voxel takes the views in order.
-// Bound by issue slots (90 % active, 49 instructions per voxel and view).  256^3 voxels and 32
-// views of 640x480, with the pre-pass: 0.766 ms; four adjacent voxels per thread with the view
-// table in shared memory took 1.115 ms (gathers of neighbouring lanes 4 voxels apart, conversions on
-// the quarter-rate unit), this mapping with the table in shared memory 0.871.  Rows below 32 voxels
-// would leave most lanes idle and take k_tsdf.
-template <int NR, bool BY_VALUE>
+// Bound by issue slots.  256^3 voxels and 32 views of 640x480, with the pre-pass: 0.77 ms; four adjacent
+// voxels per thread with the view table in shared memory took 1.12 ms (gathers of neighbouring lanes 4
+// voxels apart, conversions on the quarter-rate unit), this mapping with the table in shared memory 0.87.
+template <bool BY_VALUE>
 __global__ void __launch_bounds__(kTsdfThreads) k_tsdf_rows(float* __restrict__ F, float* __restrict__ Wt, int nx, int ny,
                                                             int64_t n_seg, int segs, TsdfParams TP,
                                                             const __grid_constant__ TsdfViews set,
@@ -153,12 +183,12 @@ __global__ void __launch_bounds__(kTsdfThreads) k_tsdf_rows(float* __restrict__ 
     const int64_t seg = (int64_t)blockIdx.x * (kTsdfThreads / 32) + (threadIdx.x >> 5);
     if (seg >= n_seg) return;
     const int64_t row = seg / segs;
-    const int i0 = (int)(seg - row * segs) * (32 * NR) + (int)lane_id();
+    const int i0 = (int)(seg - row * segs) * (32 * kLaneVox) + (int)lane_id();
     const int j = (int)(row % ny), k = (int)(row / ny);
     const float py = fmaf((float)j + 0.5f, TP.voxel, TP.oy), pz = fmaf((float)k + 0.5f, TP.voxel, TP.oz);
-    float px[NR], ms[NR], f[NR], w[NR];
+    float px[kLaneVox], ms[kLaneVox], f[kLaneVox], w[kLaneVox];
 #pragma unroll
-    for (int m = 0; m < NR; ++m) {
+    for (int m = 0; m < kLaneVox; ++m) {
         const int i = i0 + 32 * m;
         voxel_x(i, nx, TP, px[m], ms[m]);
         if (i >= nx) px[m] = __int_as_float(0x7fc00000);    // no view sees it
@@ -174,11 +204,11 @@ __global__ void __launch_bounds__(kTsdfThreads) k_tsdf_rows(float* __restrict__ 
         const float cx = cv.cx, cy = cv.cy, Wf = cv.Wf, Hf = cv.Hf;
         const uint32_t W = (uint32_t)cv.W;
         const float* __restrict__ dv = dn + cv.q0;
-        float zm[NR], d[NR];
-        uint32_t pix[NR];
-        bool ok[NR];
+        float zm[kLaneVox], d[kLaneVox];
+        uint32_t pix[kLaneVox];
+        bool ok[kLaneVox];
 #pragma unroll
-        for (int m = 0; m < NR; ++m) {
+        for (int m = 0; m < kLaneVox; ++m) {
             const float z = fmaf(ms[m], sz, fmaf(cv.R[6], px[m], rz));
             const float x = fmaf(ms[m], sx, fmaf(cv.R[0], px[m], rx)), y = fmaf(ms[m], sy, fmaf(cv.R[3], px[m], ry));
             const float iz = rcp(z);
@@ -188,12 +218,12 @@ __global__ void __launch_bounds__(kTsdfThreads) k_tsdf_rows(float* __restrict__ 
             zm[m] = z;
         }
 #pragma unroll
-        for (int m = 0; m < NR; ++m) d[m] = ok[m] ? __ldg(dv + pix[m]) : 0.f;
+        for (int m = 0; m < kLaneVox; ++m) d[m] = ok[m] ? __ldg(dv + pix[m]) : 0.f;
 #pragma unroll
-        for (int m = 0; m < NR; ++m) fuse(d[m], zm[m], ok[m], TP, f[m], w[m]);
+        for (int m = 0; m < kLaneVox; ++m) fuse(d[m], zm[m], ok[m], TP, f[m], w[m]);
     }
 #pragma unroll
-    for (int m = 0; m < NR; ++m) {
+    for (int m = 0; m < kLaneVox; ++m) {
         const int i = i0 + 32 * m;
         if (i < nx) {
             F[row * nx + i] = f[m];
@@ -211,20 +241,19 @@ static void tsdf_launch(const Launch& L, float* F, float* W, int nx, int ny, int
     constexpr int kDepthPix = kTsdfThreads * kDepthItems;
     k_tsdf_depth<BY_VALUE><<<(unsigned)((n_pix + kDepthPix - 1) / kDepthPix), kTsdfThreads, 0, L.stream>>>(
         set, table, V, n_pix, TP.min_alpha, depth, alpha, dn);
-    if (nx < 32) {
-        k_tsdf<BY_VALUE><<<(unsigned)((n_vox + kTsdfThreads - 1) / kTsdfThreads), kTsdfThreads, 0, L.stream>>>(
-            F, W, nx, ny, n_vox, TP, set, table, V, dn);
-    } else {
-        // the widest segment that leaves at most a fifth more lanes idle than single rounds do (128 x 128
-        // rows, 16 views, against the four-voxel kernel: rows of 33 voxels 59 -> 50 us, 36 53 -> 49, 50 74 ->
-        // 49, 98 114 -> 72, 130 141 -> 102, 250 232 -> 117; of 24, by k_tsdf, 49 -> 39)
-        const int rounds = (nx + 31) / 32;
-        const int NR = (rounds + 3) / 4 * 4 * 5 <= rounds * 6 ? 4 : (rounds + 1) / 2 * 2 * 5 <= rounds * 6 ? 2 : 1;
-        const int segs = (rounds + NR - 1) / NR;
+    // rows whose last segment leaves at most a sixteenth of the lanes idle are the faster form where
+    // a voxel is about a pixel or less (rows of 128, as above: 404 against 436 us; at 5 px 404 against 381,
+    // of 256 756 against 701), longer idle tails are not (112: 403 against 387; 160: 639 against 528)
+    const int segs = (nx + 32 * kLaneVox - 1) / (32 * kLaneVox);
+    if ((int64_t)segs * 32 * kLaneVox * 16 <= (int64_t)nx * 17) {
         const int64_t n_seg = n_vox / nx * segs;
-        auto* kern = NR == 4 ? k_tsdf_rows<4, BY_VALUE> : NR == 2 ? k_tsdf_rows<2, BY_VALUE> : k_tsdf_rows<1, BY_VALUE>;
-        kern<<<(unsigned)((n_seg + kTsdfThreads / 32 - 1) / (kTsdfThreads / 32)), kTsdfThreads, 0, L.stream>>>(
+        constexpr int kWarps = kTsdfThreads / 32;
+        k_tsdf_rows<BY_VALUE><<<(unsigned)((n_seg + kWarps - 1) / kWarps), kTsdfThreads, 0, L.stream>>>(
             F, W, nx, ny, n_seg, segs, TP, set, table, V, dn);
+    } else {
+        constexpr int kVox = kTsdfThreads * kLaneVox;
+        k_tsdf<BY_VALUE><<<(unsigned)((n_vox + kVox - 1) / kVox), kTsdfThreads, 0, L.stream>>>(F, W, nx, ny, n_vox, TP,
+                                                                                               set, table, V, dn);
     }
     *L.launches += 2;
 }
