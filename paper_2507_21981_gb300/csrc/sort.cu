@@ -466,10 +466,10 @@ void launch_sort(const Launch& L, uint32_t* keys, uint32_t* vals, uint32_t* keys
     *keys_out = keys;
     *vals_out = vals;
     // with a device-side count every pass runs (the output lands in the same buffer whatever
-    // the count); a host-known count of 0 or 1 is already sorted
-    if (n <= 1 && !d_n) return;
-    if (n == 0) return;
-    const bool by_view = vk && vk->bits > 0;
+    // the count); a host-known count of 0 or 1 is already sorted, but a single packed value still has to
+    // lose the view in its high bits, which its readers would take for an instance number
+    const bool by_view = vk && vk->bits > 0, packed = by_view && vk->vshift > 0;
+    if (n == 0 || (n == 1 && !d_n && !packed)) return;
     const SortPlan S(n, key_bits, by_view ? vk->bits : 0);
     sort_prepare();
     uint32_t* const hist = scratch;
@@ -482,7 +482,6 @@ void launch_sort(const Launch& L, uint32_t* keys, uint32_t* vals, uint32_t* keys
     ++*L.launches;
     uint32_t *ki = keys, *ko = keys_alt;
     uint32_t *vi = vals, *vo = vals_alt;
-    const bool packed = by_view && vk->vshift > 0;
     for (int p = 0; p < S.passes + S.vpasses; ++p) {
         // the last passes' key is the most significant one, the view, derived from the values (their
         // high bits, stripped by the last pass, or vig[value]); no keys are written for them
