@@ -38,13 +38,15 @@ struct TimedRange {
 }  // namespace
 
 // What a captured launch sequence depends on: every size that shapes a grid or a table
-// layout, and every pointer baked into a kernel argument (workspace pointers through `gen`).
+// layout, every value of the batch's tables baked into a launch (the tile bits of the keys; with two
+// view groups the second one's first tile and first count-table entry), and every pointer baked into a
+// kernel argument (workspace pointers through `gen`).  All else is read from the uploaded tables.
 struct GraphKey {
     int64_t V, K, n_nodes, dtype_mask, chunk_total, T, tiles_total, n_nv, upload_bytes, meta_bytes;
     const void *poses, *rgb, *depth, *alpha;
     uint64_t gen;
     int64_t tile_w, tile_h, exact_tile_test;
-    int64_t ng, split;
+    int64_t ng, split, split_tile, split_tab, tbits;
     const void* overlay;
     int64_t aug_on, ov_n, ov_w, ov_h;
 };
@@ -1217,7 +1219,11 @@ GraphKey make_key(const dgs_ctx* ctx, const Batch& B, const float* rgb, const fl
     k.poses = B.node_poses; k.rgb = rgb; k.depth = depth; k.alpha = alpha;
     k.gen = ctx->gen;
     k.tile_w = ctx->opt.tile_w; k.tile_h = ctx->opt.tile_h; k.exact_tile_test = ctx->opt.exact_tile_test;
-    k.ng = ctx->gng; k.split = ctx->gsplit;
+    k.ng = ctx->gng; k.split = ctx->gsplit; k.tbits = B.P.tbits;
+    if (ctx->gng == 2 && ctx->gsplit < B.V) {
+        k.split_tile = B.views[ctx->gsplit].tile_base;
+        k.split_tab = B.view_tab[ctx->gsplit];
+    }
     k.overlay = ctx->overlay;
     k.aug_on = !ctx->aug.empty(); k.ov_n = ctx->ov_n; k.ov_w = ctx->ov_w; k.ov_h = ctx->ov_h;
     return k;
