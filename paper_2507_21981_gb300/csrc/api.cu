@@ -433,7 +433,7 @@ int build_host_tables(const dgs_options& o, const dgs_node* nodes, int32_t n_nod
     if (chunk_total >= (1ll << 31)) return reject(why, DGS_ERR_INVALID_ARG, "too many Gaussians");
     // count table: per view, the chunks of its nodes in node-id order
     std::vector<int32_t> slot_node((size_t)V * K, -1);
-    std::vector<int64_t> vnode_tab((size_t)V * K, 0), view_tab(V + 1, 0);
+    std::vector<int64_t> view_tab(V + 1, 0);
     std::vector<int32_t> pmap((size_t)V * (2 * K + 1), 0);
     std::vector<std::vector<NodeView>> per_node(n_nodes);
     int64_t tab = 0, n_instances = 0;
@@ -451,13 +451,12 @@ int build_host_tables(const dgs_options& o, const dgs_node* nodes, int32_t n_nod
         int32_t pre = 0;
         for (size_t i = 0; i < present.size(); ++i) {
             const int k = present[i].first, j = present[i].second;
-            vnode_tab[(size_t)v * K + j] = tab;
             pm[i] = pre;
             pm[K + 1 + i] = j;
             pre += nd[k].nchunks;
+            per_node[k].push_back({v, j, tab});
             tab += nd[k].nchunks;
             n_instances += nd[k].n;
-            per_node[k].push_back({v, j, vnode_tab[(size_t)v * K + j]});
         }
         for (int i = (int)present.size(); i <= K; ++i) pm[i] = pre;
         for (int i = (int)present.size(); i < K; ++i) pm[K + 1 + i] = present.empty() ? 0 : present[0].second;
@@ -476,7 +475,6 @@ int build_host_tables(const dgs_options& o, const dgs_node* nodes, int32_t n_nod
     H.view_env = std::move(view_env);
     H.view_cam = std::move(view_cam);
     H.slot_node = std::move(slot_node);
-    H.vnode_tab = std::move(vnode_tab);
     H.view_tab = std::move(view_tab);
     H.pmap = std::move(pmap);
     H.nv_off = std::move(nv_off);
@@ -517,7 +515,6 @@ struct Batch {
     uint32_t* d_err = nullptr;
     const dgs_node_grads* d_grads = nullptr;
     const int32_t* d_slot = nullptr;
-    const int64_t* d_vtab = nullptr;
     const int64_t* d_viewtab = nullptr;
     const float* node_poses = nullptr;
     int64_t n_nv = 0;
@@ -559,7 +556,6 @@ int stage(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nodes, const int32_t* e
     std::vector<NodeDesc>& nd = H.nodes;
     std::vector<ViewDesc>& views = H.views;
     std::vector<int32_t>& slot_node = H.slot_node;
-    std::vector<int64_t>& vnode_tab = H.vnode_tab;
     std::vector<int64_t>& view_tab = H.view_tab;
     std::vector<int32_t>& pmap = H.pmap;
     std::vector<int32_t>& nv_off = H.nv_off;
@@ -573,7 +569,6 @@ int stage(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nodes, const int32_t* e
     const size_t o_nodes = place(sizeof(NodeDesc) * n_nodes);
     const size_t o_views = place(sizeof(ViewDesc) * V);
     const size_t o_slot = place(sizeof(int32_t) * V * K);
-    const size_t o_vtab = place(sizeof(int64_t) * V * K);
     const size_t o_nv = place(sizeof(NodeView) * std::max<size_t>(1, nv.size()));
     const size_t o_nvoff = place(sizeof(int32_t) * (n_nodes + 1));
     const size_t o_pmap = place(sizeof(int32_t) * pmap.size());
@@ -593,7 +588,6 @@ int stage(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nodes, const int32_t* e
     std::memcpy(hm + o_nodes, nd.data(), sizeof(NodeDesc) * n_nodes);
     std::memcpy(hm + o_views, views.data(), sizeof(ViewDesc) * V);
     std::memcpy(hm + o_slot, slot_node.data(), sizeof(int32_t) * V * K);
-    std::memcpy(hm + o_vtab, vnode_tab.data(), sizeof(int64_t) * V * K);
     if (!nv.empty()) std::memcpy(hm + o_nv, nv.data(), sizeof(NodeView) * nv.size());
     std::memcpy(hm + o_nvoff, nv_off.data(), sizeof(int32_t) * (n_nodes + 1));
     std::memcpy(hm + o_pmap, pmap.data(), sizeof(int32_t) * pmap.size());
@@ -605,7 +599,6 @@ int stage(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nodes, const int32_t* e
     const NodeDesc* d_nodes = reinterpret_cast<const NodeDesc*>(dm + o_nodes);
     const ViewDesc* d_views = reinterpret_cast<const ViewDesc*>(dm + o_views);
     const int32_t* d_slot = reinterpret_cast<const int32_t*>(dm + o_slot);
-    const int64_t* d_vtab = reinterpret_cast<const int64_t*>(dm + o_vtab);
     const NodeView* d_nv = reinterpret_cast<const NodeView*>(dm + o_nv);
     const int32_t* d_nvoff = reinterpret_cast<const int32_t*>(dm + o_nvoff);
     const int32_t* d_pmap = reinterpret_cast<const int32_t*>(dm + o_pmap);
@@ -646,7 +639,7 @@ int stage(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nodes, const int32_t* e
     const int tbits = bits_for((uint64_t)max_view_tiles + 1);
     B.views = std::move(views); B.view_tab = std::move(view_tab);
     B.d_nodes = d_nodes; B.d_views = d_views; B.d_nv = d_nv; B.d_nvoff = d_nvoff; B.d_pmap = d_pmap;
-    B.d_vnodes = d_vnodes; B.d_slot = d_slot; B.d_vtab = d_vtab; B.d_viewtab = d_viewtab;
+    B.d_vnodes = d_vnodes; B.d_slot = d_slot; B.d_viewtab = d_viewtab;
     B.d_counts = static_cast<uint2*>(ctx->counts.p);
     B.d_inst_off = static_cast<uint32_t*>(ctx->inst_off.p);
     B.d_pair_off = static_cast<uint64_t*>(ctx->pair_off.p);
@@ -671,17 +664,17 @@ uint64_t spin_limit_ns(const dgs_options& o) {
 void launch_front(dgs_ctx* ctx, const Batch& B, const Launch& L, Timer& tm) {
     cudaMemsetAsync(B.d_err, 0, sizeof(uint32_t) * B.call_words, L.stream);
     tm.begin(DGS_K_SETUP);
-    launch_setup_views(L, B.d_views, B.V, B.node_poses, B.d_slot, B.K, B.d_vnodes, B.d_vtab, B.d_err);
+    launch_setup_views(L, B.d_views, B.V, B.node_poses, B.d_slot, B.K, B.d_vnodes, B.d_err);
     tm.end();
     tm.begin(DGS_K_COUNT);
     if (B.batched) {
         launch_count(L, B.dtype_mask, B.d_nodes, B.n_nodes, B.d_views, B.d_vnodes, B.K, B.d_nv, B.d_nvoff,
-                     (int)B.chunk_total, B.P, 0, B.V, true, nullptr, 0, B.d_counts);
+                     (int)B.chunk_total, B.P, 0, B.V, true, nullptr, 0, 0, B.d_counts);
     } else {
         for (int v = 0; v < B.V; ++v)
             launch_count(L, B.dtype_mask, B.d_nodes, B.n_nodes, B.d_views, B.d_vnodes, B.K, B.d_nv, B.d_nvoff,
                          (int)B.chunk_total, B.P, v, v + 1, false, B.d_pmap + (size_t)v * (2 * B.K + 1),
-                         B.view_tab[v + 1] - B.view_tab[v], B.d_counts);
+                         B.view_tab[v], B.view_tab[v + 1] - B.view_tab[v], B.d_counts);
     }
     tm.end();
     tm.begin(DGS_K_SCAN);
@@ -873,7 +866,8 @@ void enqueue_lists(dgs_ctx* ctx, ListBufs& lb, const Batch& B, const Launch& L, 
     Pe.vkey = plan.depth_bits > kZBits;
     tm.begin(DGS_K_EMIT);
     launch_emit(L, B.dtype_mask, B.d_nodes, B.n_nodes, B.d_views, B.d_vnodes, K, B.d_nv, B.d_nvoff, (int)B.chunk_total,
-                Pe, v0, v1, B.batched, B.d_pmap + (size_t)v0 * (2 * K + 1), B.view_tab[v0 + 1] - B.view_tab[v0],
+                Pe, v0, v1, B.batched, B.d_pmap + (size_t)v0 * (2 * K + 1), B.view_tab[v0],
+                B.view_tab[v0 + 1] - B.view_tab[v0],
                 B.d_counts, B.d_inst_off, inst_base, rec, info, u32(lb.dkey0), u32(lb.ival0), u32(lb.ntile),
                 const_cast<uint32_t*>(vk.vig));
     tm.end();

@@ -292,7 +292,8 @@ void launch_tile_scan(const Launch& L, const uint32_t* order, const uint32_t* nt
     ++*L.launches;
 }
 
-ListPlan plan_lists(uint32_t n_inst, uint32_t n_pairs, int n_views, int tbits, int64_t n_tiles, bool separate_view_key) {
+ListPlan plan_lists(uint32_t n_inst, uint32_t n_pairs, int n_views, int tbits, int64_t n_tiles, bool separate_view_key,
+                    bool compact) {
     ListPlan p;
     int vb = 0;
     while (vb < 31 && (1ll << vb) < n_views) ++vb;
@@ -300,10 +301,12 @@ ListPlan plan_lists(uint32_t n_inst, uint32_t n_pairs, int n_views, int tbits, i
     else p.view_bits = vb;
     size_t at = 0;
     auto take = [&](size_t words) { const size_t r = at; at += (words + 3) & ~size_t(3); return r; };
-    p.depth = take(sort_scratch_words(n_inst, p.depth_bits, p.view_bits));
+    const size_t depth = sort_scratch_words(n_inst, p.depth_bits, p.view_bits, compact);
+    const size_t tile = sort_scratch_words(n_pairs, tbits, 0, compact);
+    p.depth = p.tile = take(compact ? std::max(depth, tile) : depth);
+    if (!compact) p.tile = take(tile);
     p.tscan = take(tile_scan_words(n_inst));
-    p.tile = take(sort_scratch_words(n_pairs, tbits, 0));
-    p.order = take(kOrderWords);
+    if (!compact) p.order = take(kOrderWords);
     p.ranges = take(2 * (size_t)std::max<int64_t>(n_tiles, 1));
     p.words = at;
     return p;

@@ -95,10 +95,9 @@ struct VNode {
     float Ml[12];         // trailing parts: camera_from_node = M + Ml to about 2^-48
     float o[3];           // camera centre in the node frame
     int32_t node;         // -1 = empty slot
-    int64_t tab;          // count-table index of the node's first chunk in this view
-    int64_t pad[3];       // 144 bytes: the emission reads the transform in quads; at a stride of 128 the
-                          // count pass, whose lanes read 32 transforms each, takes 1.4x as long
-};
+};                        // 112 bytes: the emission reads the transform in quads; at a stride of 128 the
+                          // count pass, whose lanes read 32 transforms each, takes 1.4x as long (128
+                          // views: 430 us, 306 at a stride of 144, 300 at 112)
 static_assert(sizeof(ViewDesc) % 16 == 0 && sizeof(VNode) % 16 == 0, "read in 16-byte quads");
 
 // Error-free transformations in binary32 (Knuth's TwoSum; TwoProduct by a fused multiply-add):
@@ -200,7 +199,6 @@ struct HostTables {
     std::vector<ViewDesc> views;
     std::vector<int> view_env, view_cam;
     std::vector<int32_t> slot_node;    // [V*K] node drawn in slot j of view v's env (-1 = empty)
-    std::vector<int64_t> vnode_tab;    // [V*K] count-table entry of (view, slot)'s first chunk
     std::vector<int64_t> view_tab;     // [V+1] first count-table entry of each view; [V] = T
     std::vector<int32_t> pmap;         // [V*(2K+1)] plain mode: per view, chunk prefix and slot of
                                        // each present node in node-id order
@@ -461,13 +459,13 @@ struct Launch {
 };
 
 void launch_setup_views(const Launch& L, const ViewDesc* views, int n_views, const float* node_poses,
-                        const int32_t* view_slots_node, int K, VNode* vnodes, const int64_t* vnode_tab,
-                        uint32_t* err);
+                        const int32_t* view_slots_node, int K, VNode* vnodes, uint32_t* err);
 
+// (plain mode: the view's chunks by node, its first count-table entry and its number of entries)
 void launch_count(const Launch& L, int dtype_mask, const NodeDesc* nodes, int n_nodes, const ViewDesc* views,
                   const VNode* vnodes, int K, const NodeView* node_views, const int32_t* node_view_off,
                   int n_chunks_total, const Params& P, int v0, int v1, bool batched, const int32_t* view_chunk_nodes,
-                  int64_t view_chunks, uint2* counts);
+                  int64_t view_first, int64_t view_chunks, uint2* counts);
 
 // Exclusive scan of the count table: inst_off[n + 1] (32 bits, wrapping), pair_off[n + 1].  scratch:
 // scan_words(n) words, 16-byte aligned and zero on entry; *scan_total(scratch) receives the 64-bit
@@ -483,7 +481,7 @@ void launch_scan(const Launch& L, const uint2* counts, int64_t n, uint32_t* inst
 void launch_emit(const Launch& L, int dtype_mask, const NodeDesc* nodes, int n_nodes, const ViewDesc* views,
                  const VNode* vnodes, int K, const NodeView* node_views, const int32_t* node_view_off,
                  int n_chunks_total, const Params& P, int v0, int v1, bool batched, const int32_t* view_chunk_nodes,
-                 int64_t view_chunks, const uint2* counts, const uint32_t* inst_off, uint32_t inst_base,
+                 int64_t view_first, int64_t view_chunks, const uint2* counts, const uint32_t* inst_off, uint32_t inst_base,
                  Record* records, InstInfo* info, uint32_t* dkey, uint32_t* ival, uint32_t* ntile, uint32_t* vig);
 
 // Bounded waits of the sort: the look-back spin limit, and a test of it (mute_part: the
@@ -492,6 +490,7 @@ struct SortCtl {
     uint64_t spin_ns = 1000000000ull;
     uint32_t mute_part = 0xFFFFFFFFu;
     bool runs = false;    // neighbouring keys share their high digits (histogram by runs)
+    bool compact = false; // the passes share one look-back region, cleared before each (less scratch)
 };
 
 // The depth sort's most significant key: the view of each instance within its view group.
@@ -513,9 +512,9 @@ struct ViewKey {
 // are sized for.  *keys_out / *vals_out receive the buffers holding the result.  A look-back
 // wait that runs out sets kErrTimeout in err (the output is then invalid).  With vk (bits > 0)
 // the values are then sorted stably by their view, as a more significant key; no sorted keys
-// are then written (*keys_out is null).  scratch: sort_scratch_words(n, key_bits, vk ? vk->bits : 0)
-// words, zero on entry.
-size_t sort_scratch_words(uint32_t n, int key_bits, int view_bits);
+// are then written (*keys_out is null).  scratch: sort_scratch_words(n, key_bits, vk ? vk->bits : 0,
+// ctl.compact) words, zero on entry.
+size_t sort_scratch_words(uint32_t n, int key_bits, int view_bits, bool compact = false);
 void launch_sort(const Launch& L, uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt,
                  uint32_t n, int key_bits, uint32_t* scratch, uint32_t* err, uint32_t** keys_out,
                  uint32_t** vals_out, const uint32_t* d_n = nullptr, SortCtl ctl = SortCtl{},
@@ -544,7 +543,10 @@ struct ListPlan {
     int view_bits = 0;                  // bits of a separate view key
     size_t depth = 0, tscan = 0, tile = 0, order = 0, ranges = 0, words = 0;
 };
-ListPlan plan_lists(uint32_t n_inst, uint32_t n_pairs, int n_views, int tbits, int64_t n_tiles, bool separate_view_key);
+// compact: the sorts share one region (to be cleared again before the tile sort), and there is none for
+// a tile order.
+ListPlan plan_lists(uint32_t n_inst, uint32_t n_pairs, int n_views, int tbits, int64_t n_tiles, bool separate_view_key,
+                    bool compact = false);
 // Words that hold the plan of any group of at most these sizes, whatever its views and tile bits.
 size_t list_scratch_bound(uint32_t n_inst, uint32_t n_pairs, int64_t n_tiles);
 

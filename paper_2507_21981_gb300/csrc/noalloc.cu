@@ -58,17 +58,19 @@ cudaError_t scratch_address(unsigned char** out) {
 
 struct Carver {
     unsigned char* base;
+    size_t align = 256;
     size_t used = 0;
     bool ok = true;
     template <class T>
-    T* take(size_t count) {
-        size_t at = (used + 255) / 256 * 256;
+    void take(T*& p, size_t count) {
+        size_t at = (used + align - 1) / align * align;
         size_t bytes = sizeof(T) * std::max<size_t>(count, 1);
-        if (at + bytes > kScratchBytes) { ok = false; return nullptr; }
+        if (at + bytes > kScratchBytes) { ok = false; return; }
         used = at + bytes;
-        return reinterpret_cast<T*>(base + at);
+        p = reinterpret_cast<T*>(base + at);
     }
 };
+constexpr size_t kTightAlign = 32;     // where the arrays do not fit at 256 bytes: one sector
 
 int bits_for_tiles(uint64_t n) {
     int b = 0;
@@ -100,7 +102,6 @@ extern "C" int dgs_render_noalloc(const dgs_options* opt, const dgs_node* nodes,
     const std::vector<NodeDesc>& nd = H.nodes;
     const std::vector<ViewDesc>& views = H.views;
     const std::vector<int32_t>& slot_node = H.slot_node;
-    const std::vector<int64_t>& vnode_tab = H.vnode_tab;
     const std::vector<int64_t>& view_tab = H.view_tab;
     const std::vector<int32_t>& nv_off = H.nv_off;
     const std::vector<NodeView>& nv = H.nv;
@@ -110,21 +111,33 @@ extern "C" int dgs_render_noalloc(const dgs_options* opt, const dgs_node* nodes,
     // ---------------------------------------------------------------- phase 1 scratch
     unsigned char* base = nullptr;
     if (scratch_address(&base) != cudaSuccess) return DGS_ERR_CUDA;
-    Carver cv{base};
-    NodeDesc* d_nodes = cv.take<NodeDesc>(n_nodes);
-    ViewDesc* d_views = cv.take<ViewDesc>(V);
-    int32_t* d_slot = cv.take<int32_t>((size_t)V * K);
-    int64_t* d_vtab = cv.take<int64_t>((size_t)V * K);
-    NodeView* d_nv = cv.take<NodeView>(nv.size());
-    int32_t* d_nvoff = cv.take<int32_t>(n_nodes + 1);
-    int64_t* d_viewtab = cv.take<int64_t>(V + 1);
-    VNode* d_vnodes = cv.take<VNode>((size_t)V * K);
-    uint32_t* d_err = cv.take<uint32_t>(kErrBlockBytes / 4);
-    uint2* d_counts = cv.take<uint2>(T);
-    uint32_t* d_inst_off = cv.take<uint32_t>(T + 1);
-    uint64_t* d_pair_off = cv.take<uint64_t>(T + 1);
-    uint32_t* d_scan = cv.take<uint32_t>(scan_words(T));
-    uint64_t* d_rb = cv.take<uint64_t>(2 * (V + 1) + 1);
+    NodeDesc* d_nodes = nullptr;
+    ViewDesc* d_views = nullptr;
+    int32_t *d_slot = nullptr, *d_nvoff = nullptr;
+    NodeView* d_nv = nullptr;
+    int64_t* d_viewtab = nullptr;
+    VNode* d_vnodes = nullptr;
+    uint32_t *d_err = nullptr, *d_inst_off = nullptr, *d_scan = nullptr;
+    uint2* d_counts = nullptr;
+    uint64_t *d_pair_off = nullptr, *d_rb = nullptr;
+    auto carve1 = [&](Carver c) {
+        c.take(d_nodes, n_nodes);
+        c.take(d_views, V);
+        c.take(d_slot, (size_t)V * K);
+        c.take(d_nv, nv.size());
+        c.take(d_nvoff, n_nodes + 1);
+        c.take(d_viewtab, V + 1);
+        c.take(d_vnodes, (size_t)V * K);
+        c.take(d_err, kErrBlockBytes / 4);
+        c.take(d_counts, T);
+        c.take(d_inst_off, T + 1);
+        c.take(d_pair_off, T + 1);
+        c.take(d_scan, scan_words(T));
+        c.take(d_rb, 2 * (V + 1) + 1);
+        return c;
+    };
+    Carver cv = carve1(Carver{base});
+    if (!cv.ok) cv = carve1(Carver{base, kTightAlign});
     if (!cv.ok) return DGS_ERR_CAPACITY;
 
 #define NA_CUDA(x) do { if ((x) != cudaSuccess) return DGS_ERR_CUDA; } while (0)
@@ -132,7 +145,6 @@ extern "C" int dgs_render_noalloc(const dgs_options* opt, const dgs_node* nodes,
     NA_CUDA(cudaMemcpyAsync(d_nodes, nd.data(), sizeof(NodeDesc) * n_nodes, cudaMemcpyHostToDevice, stream));
     NA_CUDA(cudaMemcpyAsync(d_views, views.data(), sizeof(ViewDesc) * V, cudaMemcpyHostToDevice, stream));
     NA_CUDA(cudaMemcpyAsync(d_slot, slot_node.data(), sizeof(int32_t) * V * K, cudaMemcpyHostToDevice, stream));
-    NA_CUDA(cudaMemcpyAsync(d_vtab, vnode_tab.data(), sizeof(int64_t) * V * K, cudaMemcpyHostToDevice, stream));
     if (!nv.empty()) NA_CUDA(cudaMemcpyAsync(d_nv, nv.data(), sizeof(NodeView) * nv.size(), cudaMemcpyHostToDevice, stream));
     NA_CUDA(cudaMemcpyAsync(d_nvoff, nv_off.data(), sizeof(int32_t) * (n_nodes + 1), cudaMemcpyHostToDevice, stream));
     NA_CUDA(cudaMemcpyAsync(d_viewtab, view_tab.data(), sizeof(int64_t) * (V + 1), cudaMemcpyHostToDevice, stream));
@@ -142,9 +154,9 @@ extern "C" int dgs_render_noalloc(const dgs_options* opt, const dgs_node* nodes,
     P.err = d_err;
     int64_t launches = 0;
     Launch L{stream, &launches};
-    launch_setup_views(L, d_views, V, node_poses, d_slot, K, d_vnodes, d_vtab, d_err);
+    launch_setup_views(L, d_views, V, node_poses, d_slot, K, d_vnodes, d_err);
     launch_count(L, dtype_mask, d_nodes, n_nodes, d_views, d_vnodes, K, d_nv, d_nvoff, (int)chunk_total, P, 0, V, true,
-                 nullptr, 0, d_counts);
+                 nullptr, 0, 0, d_counts);
     NA_CUDA(cudaMemsetAsync(d_scan, 0, sizeof(uint32_t) * scan_words(T), stream));
     launch_scan(L, d_counts, T, d_inst_off, d_pair_off, d_scan, d_err, SortCtl{}.spin_ns);
     // one view group: read back the grand totals and the error word
@@ -165,20 +177,6 @@ extern "C" int dgs_render_noalloc(const dgs_options* opt, const dgs_node* nodes,
 
     // ---------------------------------------------------------------- phase 2 scratch
     const uint64_t ni = std::max<uint64_t>(n_vis, 1), np = std::max<uint64_t>(n_pairs, 1);
-    Record* d_rec = cv.take<Record>(ni);
-    InstInfo* d_info = cv.take<InstInfo>(ni);
-    uint32_t* d_dk0 = cv.take<uint32_t>(ni);
-    uint32_t* d_iv0 = cv.take<uint32_t>(ni);
-    uint32_t* d_dk1 = cv.take<uint32_t>(ni);
-    uint32_t* d_iv1 = cv.take<uint32_t>(ni);
-    uint32_t* d_ntile = cv.take<uint32_t>(ni);
-    uint32_t* d_poff = cv.take<uint32_t>(ni + 1);
-    uint32_t* d_k0 = cv.take<uint32_t>(np);
-    uint32_t* d_v0 = cv.take<uint32_t>(np);
-    uint32_t* d_k1 = cv.take<uint32_t>(np);
-    uint32_t* d_v1 = cv.take<uint32_t>(np);
-    uint32_t* d_total = cv.take<uint32_t>(1);
-    if (!cv.ok) return DGS_ERR_CAPACITY;
     // tile keys: view << tbits | tile in view, as in dgs_render with one view group
     int64_t max_view_tiles = 1;
     for (const ViewDesc& vd : views) max_view_tiles = std::max<int64_t>(max_view_tiles, (int64_t)vd.tiles_x * vd.tiles_y);
@@ -186,9 +184,27 @@ extern "C" int dgs_render_noalloc(const dgs_options* opt, const dgs_node* nodes,
     if (tbits > kTileBits || tiles_total > kMaxGroupTiles || (int64_t)V >= (1ll << (kTileBits - tbits)))
         return DGS_ERR_CAPACITY;
     // depth-ordered tile lists, as in dgs_render with one view group
-    const ListPlan plan = plan_lists((uint32_t)n_vis, (uint32_t)n_pairs, V, tbits, tiles_total, false);
-    uint32_t* d_scratch = cv.take<uint32_t>(plan.words);
-    if (!cv.ok) return DGS_ERR_CAPACITY;
+    Record* d_rec = nullptr;
+    InstInfo* d_info = nullptr;
+    uint32_t *d_dk0 = nullptr, *d_iv0 = nullptr, *d_dk1 = nullptr, *d_iv1 = nullptr, *d_ntile = nullptr, *d_poff = nullptr;
+    uint32_t *d_k0 = nullptr, *d_v0 = nullptr, *d_k1 = nullptr, *d_v1 = nullptr, *d_total = nullptr, *d_scratch = nullptr;
+    ListPlan plan;
+    auto carve2 = [&](Carver c, bool compact) {
+        plan = plan_lists((uint32_t)n_vis, (uint32_t)n_pairs, V, tbits, tiles_total, false, compact);
+        c.take(d_rec, ni);
+        c.take(d_info, ni);
+        for (uint32_t** p : {&d_dk0, &d_iv0, &d_dk1, &d_iv1, &d_ntile}) c.take(*p, ni);
+        c.take(d_poff, ni + 1);
+        for (uint32_t** p : {&d_k0, &d_v0, &d_k1, &d_v1}) c.take(*p, np);
+        c.take(d_total, 1);
+        c.take(d_scratch, plan.words);
+        return c.ok;
+    };
+    // the sorts' scratch costs up to 0.7 bytes a pair; a batch that does not fit with it clears one
+    // region before every pass instead
+    const bool compact = !carve2(cv, false);
+    cv.align = kTightAlign;
+    if (compact && !carve2(cv, true)) return DGS_ERR_CAPACITY;
     uint2* d_ranges = reinterpret_cast<uint2*>(d_scratch + plan.ranges);
     NA_CUDA(cudaMemsetAsync(d_scratch, 0, sizeof(uint32_t) * plan.words, stream));
     // a separate view key of the depth sort: packed into the instance numbers where both fit in 32
@@ -208,10 +224,11 @@ extern "C" int dgs_render_noalloc(const dgs_options* opt, const dgs_node* nodes,
     P.vshift = vk.vshift;
     P.vkey = plan.depth_bits > kZBits;
     launch_emit(L, dtype_mask, d_nodes, n_nodes, d_views, d_vnodes, K, d_nv, d_nvoff, (int)chunk_total, P, 0, V, true,
-                nullptr, 0, d_counts, d_inst_off, 0u, d_rec, d_info, d_dk0, d_iv0, d_ntile, vk.vig ? d_vig : nullptr);
+                nullptr, 0, 0, d_counts, d_inst_off, 0u, d_rec, d_info, d_dk0, d_iv0, d_ntile, vk.vig ? d_vig : nullptr);
     uint32_t *dk, *order, *tk, *tv;
     SortCtl depth_ctl;
     depth_ctl.runs = true;
+    depth_ctl.compact = compact;
     launch_sort(L, d_dk0, d_iv0, d_dk1, d_iv1, (uint32_t)n_vis, plan.depth_bits, d_scratch + plan.depth, d_err,
                 &dk, &order, nullptr, depth_ctl, &vk);
     launch_tile_scan(L, order, d_ntile, (uint32_t)n_vis, nullptr, d_poff, d_scratch + plan.tscan, (uint32_t)n_pairs,
@@ -219,6 +236,10 @@ extern "C" int dgs_render_noalloc(const dgs_options* opt, const dgs_node* nodes,
     launch_pairs(L, d_views, K, order, d_poff, d_rec, d_info, (uint32_t)n_vis, nullptr, P, d_k0, d_v0, (uint32_t)n_pairs);
     SortCtl tile_ctl;
     tile_ctl.runs = true;
+    tile_ctl.compact = compact;
+    if (compact)
+        NA_CUDA(cudaMemsetAsync(d_scratch + plan.tile, 0,
+                                sizeof(uint32_t) * sort_scratch_words((uint32_t)n_pairs, tbits, 0, true), stream));
     launch_sort(L, d_k0, d_v0, d_k1, d_v1, (uint32_t)n_pairs, tbits, d_scratch + plan.tile, d_err, &tk, &tv, d_total,
                 tile_ctl);
     launch_ranges(L, tk, (uint32_t)n_pairs, d_ranges, (int)tiles_total, d_total, d_views, V, P);

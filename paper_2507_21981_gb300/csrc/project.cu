@@ -41,14 +41,13 @@ __device__ __forceinline__ void dot_hi_lo(const float* a, const float* b, int n,
 }
 __global__ void k_setup_views(const ViewDesc* __restrict__ views, int n_views, const float* __restrict__ poses,
                               const int32_t* __restrict__ slot_node, int K, VNode* __restrict__ vnodes,
-                              const int64_t* __restrict__ vnode_tab, uint32_t* err) {
+                              uint32_t* err) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_views * K) return;
     const int v = i / K, j = i % K;
     const ViewDesc& vd = views[v];
     VNode out;
     out.node = slot_node[i];
-    out.tab = vnode_tab[i];
     const float* P = poses + ((int64_t)vd.env * K + j) * 12;
     float R[9], t[3];
     bool bad = false;
@@ -709,7 +708,7 @@ __global__ void __launch_bounds__(kCountWarps * 32) k_count_batched(const NodeDe
 template <int DT>
 __global__ void __launch_bounds__(kCountWarps * 32) k_count_plain(const NodeDesc* __restrict__ nodes,
         const ViewDesc* __restrict__ views, const VNode* __restrict__ vnodes, int K, Params P, int v,
-        const int32_t* __restrict__ pmap, int n_view_chunks, uint2* counts) {
+        const int32_t* __restrict__ pmap, int64_t view_first, int n_view_chunks, uint2* counts) {
     __shared__ WarpWork ww[kCountWarps];
     const int w = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     if (w >= n_view_chunks) return;
@@ -725,7 +724,7 @@ __global__ void __launch_bounds__(kCountWarps * 32) k_count_plain(const NodeDesc
     bool valid;
     stage_geometry<DT>(nd, c, lane, W, g, valid);
     const ChunkBound cb = chunk_bound(g, valid);
-    const NodeView one{v, slot, vnodes[v * K + slot].tab};
+    const NodeView one{v, slot, view_first + pmap[lo]};
     process_chunk<false, DT>(nd, c, lane, &one, 1, v, v + 1, views, vnodes, K, P, g, valid, cb, W, nullptr, counts,
                              nullptr, 0, EmitOut{});
 }
@@ -755,7 +754,7 @@ __global__ void __launch_bounds__(kEmitWarps * 32, 5) k_emit_batched(const NodeD
 template <int DT>
 __global__ void __launch_bounds__(kEmitWarps * 32, 5) k_emit_plain(const NodeDesc* __restrict__ nodes,
         const ViewDesc* __restrict__ views, const VNode* __restrict__ vnodes, int K, Params P, int v,
-        const int32_t* __restrict__ pmap, int n_view_chunks, const uint2* __restrict__ counts,
+        const int32_t* __restrict__ pmap, int64_t view_first, int n_view_chunks, const uint2* __restrict__ counts,
         const uint32_t* __restrict__ inst_off, uint32_t inst_base, EmitOut out) {
     __shared__ WarpWork ww[kEmitWarps];
     __shared__ alignas(16) float shc[kEmitWarps][kChunk * kShStride];
@@ -769,7 +768,7 @@ __global__ void __launch_bounds__(kEmitWarps * 32, 5) k_emit_plain(const NodeDes
     const NodeDesc& nd = nodes[vnodes[v * K + slot].node];
     if (nd.dtype != DT) return;
     const int c = w - pmap[lo];
-    const NodeView one{v, slot, vnodes[v * K + slot].tab};
+    const NodeView one{v, slot, view_first + pmap[lo]};
     process_chunk<true, DT>(nd, c, lane, &one, 1, v, v + 1, views, vnodes, K, P, Gauss{}, false, ChunkBound{}, W,
                             shc[wib], const_cast<uint2*>(counts), inst_off, inst_base, out);
 }
@@ -924,7 +923,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const uint2* __restrict__
 template <int DT>
 void count_launch(const Launch& L, const NodeDesc* nodes, int n_nodes, const ViewDesc* views, const VNode* vnodes, int K,
                   const NodeView* nv, const int32_t* nv_off, int n_chunks, const Params& P, int v0, int v1,
-                  bool batched, const int32_t* pmap, int64_t view_chunks, uint2* counts) {
+                  bool batched, const int32_t* pmap, int64_t view_first, int64_t view_chunks, uint2* counts) {
     if (batched) {
         const int blocks = (int)(((int64_t)n_chunks + kCountWarps - 1) / kCountWarps);
         if (blocks == 0) return;
@@ -933,7 +932,7 @@ void count_launch(const Launch& L, const NodeDesc* nodes, int n_nodes, const Vie
     } else {
         const int blocks = (int)((view_chunks + kCountWarps - 1) / kCountWarps);
         if (blocks == 0) return;
-        k_count_plain<DT><<<blocks, kCountWarps * 32, 0, L.stream>>>(nodes, views, vnodes, K, P, v0, pmap, (int)view_chunks, counts);
+        k_count_plain<DT><<<blocks, kCountWarps * 32, 0, L.stream>>>(nodes, views, vnodes, K, P, v0, pmap, view_first, (int)view_chunks, counts);
     }
     ++*L.launches;
 }
@@ -941,7 +940,7 @@ void count_launch(const Launch& L, const NodeDesc* nodes, int n_nodes, const Vie
 template <int DT>
 void emit_launch(const Launch& L, const NodeDesc* nodes, int n_nodes, const ViewDesc* views, const VNode* vnodes, int K,
                  const NodeView* nv, const int32_t* nv_off, int n_chunks, const Params& P, int v0, int v1, bool batched,
-                 const int32_t* pmap, int64_t view_chunks, const uint2* counts, const uint32_t* inst_off,
+                 const int32_t* pmap, int64_t view_first, int64_t view_chunks, const uint2* counts, const uint32_t* inst_off,
                  uint32_t inst_base, const EmitOut& out) {
     if (batched) {
         const int blocks = (int)(((int64_t)n_chunks + kEmitWarps - 1) / kEmitWarps);
@@ -951,7 +950,7 @@ void emit_launch(const Launch& L, const NodeDesc* nodes, int n_nodes, const View
     } else {
         const int blocks = (int)((view_chunks + kEmitWarps - 1) / kEmitWarps);
         if (blocks == 0) return;
-        k_emit_plain<DT><<<blocks, kEmitWarps * 32, 0, L.stream>>>(nodes, views, vnodes, K, P, v0, pmap, (int)view_chunks,
+        k_emit_plain<DT><<<blocks, kEmitWarps * 32, 0, L.stream>>>(nodes, views, vnodes, K, P, v0, pmap, view_first, (int)view_chunks,
                                                                    counts, inst_off, inst_base, out);
     }
     ++*L.launches;
@@ -960,43 +959,43 @@ void emit_launch(const Launch& L, const NodeDesc* nodes, int n_nodes, const View
 }  // namespace
 
 void launch_setup_views(const Launch& L, const ViewDesc* views, int n_views, const float* node_poses,
-                        const int32_t* slot_node, int K, VNode* vnodes, const int64_t* vnode_tab, uint32_t* err) {
+                        const int32_t* slot_node, int K, VNode* vnodes, uint32_t* err) {
     const int n = n_views * K;
     if (n == 0) return;
-    k_setup_views<<<(n + 127) / 128, 128, 0, L.stream>>>(views, n_views, node_poses, slot_node, K, vnodes, vnode_tab, err);
+    k_setup_views<<<(n + 127) / 128, 128, 0, L.stream>>>(views, n_views, node_poses, slot_node, K, vnodes, err);
     ++*L.launches;
 }
 
 void launch_count(const Launch& L, int dtype_mask, const NodeDesc* nodes, int n_nodes, const ViewDesc* views,
                   const VNode* vnodes, int K, const NodeView* node_views, const int32_t* node_view_off,
                   int n_chunks_total, const Params& P, int v0, int v1, bool batched, const int32_t* pmap,
-                  int64_t view_chunks, uint2* counts) {
+                  int64_t view_first, int64_t view_chunks, uint2* counts) {
     if (dtype_mask & (1 << DGS_F32))
         count_launch<DGS_F32>(L, nodes, n_nodes, views, vnodes, K, node_views, node_view_off, n_chunks_total, P, v0, v1,
-                              batched, pmap, view_chunks, counts);
+                              batched, pmap, view_first, view_chunks, counts);
     if (dtype_mask & (1 << DGS_BF16))
         count_launch<DGS_BF16>(L, nodes, n_nodes, views, vnodes, K, node_views, node_view_off, n_chunks_total, P, v0, v1,
-                               batched, pmap, view_chunks, counts);
+                               batched, pmap, view_first, view_chunks, counts);
     if (dtype_mask & (1 << DGS_F16))
         count_launch<DGS_F16>(L, nodes, n_nodes, views, vnodes, K, node_views, node_view_off, n_chunks_total, P, v0, v1,
-                              batched, pmap, view_chunks, counts);
+                              batched, pmap, view_first, view_chunks, counts);
 }
 
 void launch_emit(const Launch& L, int dtype_mask, const NodeDesc* nodes, int n_nodes, const ViewDesc* views,
                  const VNode* vnodes, int K, const NodeView* node_views, const int32_t* node_view_off,
                  int n_chunks_total, const Params& P, int v0, int v1, bool batched, const int32_t* pmap,
-                 int64_t view_chunks, const uint2* counts, const uint32_t* inst_off, uint32_t inst_base,
+                 int64_t view_first, int64_t view_chunks, const uint2* counts, const uint32_t* inst_off, uint32_t inst_base,
                  Record* records, InstInfo* info, uint32_t* dkey, uint32_t* ival, uint32_t* ntile, uint32_t* vig) {
     const EmitOut out{records, info, dkey, ival, ntile, vig};
     if (dtype_mask & (1 << DGS_F32))
         emit_launch<DGS_F32>(L, nodes, n_nodes, views, vnodes, K, node_views, node_view_off, n_chunks_total, P, v0, v1,
-                             batched, pmap, view_chunks, counts, inst_off, inst_base, out);
+                             batched, pmap, view_first, view_chunks, counts, inst_off, inst_base, out);
     if (dtype_mask & (1 << DGS_BF16))
         emit_launch<DGS_BF16>(L, nodes, n_nodes, views, vnodes, K, node_views, node_view_off, n_chunks_total, P, v0, v1,
-                              batched, pmap, view_chunks, counts, inst_off, inst_base, out);
+                              batched, pmap, view_first, view_chunks, counts, inst_off, inst_base, out);
     if (dtype_mask & (1 << DGS_F16))
         emit_launch<DGS_F16>(L, nodes, n_nodes, views, vnodes, K, node_views, node_view_off, n_chunks_total, P, v0, v1,
-                             batched, pmap, view_chunks, counts, inst_off, inst_base, out);
+                             batched, pmap, view_first, view_chunks, counts, inst_off, inst_base, out);
 }
 
 size_t scan_words(int64_t n) { return 8 + 4 * (size_t)((n + kScanTile - 1) / kScanTile); }

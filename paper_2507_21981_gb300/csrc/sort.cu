@@ -422,7 +422,7 @@ struct SortPlan {
     int passes, D, last, vpasses, vD, vlast;
     uint32_t parts;
     size_t counters, status[8], words;
-    SortPlan(uint32_t n, int key_bits, int view_bits) {
+    SortPlan(uint32_t n, int key_bits, int view_bits, bool compact) {
         const int bits = std::max(1, key_bits);
         passes = sort_passes(bits);
         D = (bits + passes - 1) / passes;
@@ -432,13 +432,15 @@ struct SortPlan {
         vlast = vpasses ? view_bits - vD * (vpasses - 1) : 0;
         parts = (n + kTile - 1) / kTile;
         counters = (size_t)kMaxR * (passes + vpasses);
-        words = counters + 16;
+        const size_t first = counters + 16;
+        words = first;
         for (int p = 0; p < passes + vpasses; ++p) {
-            status[p] = words;
-            words += (size_t)parts << digit_bits(p);
+            status[p] = compact ? first : words;
+            words = std::max(words, status[p] + status_words(p));
         }
         words = (words + 3) & ~size_t(3);
     }
+    size_t status_words(int p) const { return (size_t)parts << digit_bits(p); }
     int digit_bits(int p) const {
         return p < passes ? (p == passes - 1 ? last : D) : (p - passes == vpasses - 1 ? vlast : vD);
     }
@@ -446,7 +448,9 @@ struct SortPlan {
 
 }  // namespace
 
-size_t sort_scratch_words(uint32_t n, int key_bits, int view_bits) { return SortPlan(n, key_bits, view_bits).words; }
+size_t sort_scratch_words(uint32_t n, int key_bits, int view_bits, bool compact) {
+    return SortPlan(n, key_bits, view_bits, compact).words;
+}
 
 void sort_prepare() {
     static bool attr_set = false;
@@ -470,7 +474,7 @@ void launch_sort(const Launch& L, uint32_t* keys, uint32_t* vals, uint32_t* keys
     // lose the view in its high bits, which its readers would take for an instance number
     const bool by_view = vk && vk->bits > 0, packed = by_view && vk->vshift > 0;
     if (n == 0 || (n == 1 && !d_n && !packed)) return;
-    const SortPlan S(n, key_bits, by_view ? vk->bits : 0);
+    const SortPlan S(n, key_bits, by_view ? vk->bits : 0, ctl.compact);
     sort_prepare();
     uint32_t* const hist = scratch;
     uint32_t* const counters = scratch + S.counters;
@@ -491,6 +495,8 @@ void launch_sort(const Launch& L, uint32_t* keys, uint32_t* vals, uint32_t* keys
                                                                          : onesweep_for<kKeysGather>(Dp);
         uint32_t* kw = by_view && p >= S.passes - 1 ? nullptr : ko;
         const uint32_t vmask = packed && p == S.passes + S.vpasses - 1 ? (1u << vk->vshift) - 1u : 0xFFFFFFFFu;
+        if (ctl.compact && p > 0)
+            cudaMemsetAsync(scratch + S.status[p], 0, sizeof(uint32_t) * S.status_words(p), L.stream);
         fn<<<S.parts, kThreads, kSmem, L.stream>>>(ki, vi, kw, vo, n, d_n, shift, hist + p * kMaxR,
                                                    scratch + S.status[p], counters + p, err, ctl.spin_ns,
                                                    p == 0 ? ctl.mute_part : 0xFFFFFFFFu, view ? vk->vig : nullptr,
