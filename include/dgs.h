@@ -507,8 +507,10 @@ int dgs_lidar_build(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nodes, void* 
  *   out_d, out_a                  DEVICE FP32 [n_sensors*n_dirs], sensor-major (sensors, dirs and the
  *                                 outputs may be NULL when n_sensors = 0: nothing is traced)
  * Work is queued on `stream`; the call synchronises it before returning (device-side pose
- * validation is reported as DGS_ERR_INVALID_ARG).  Every ray is traced by itself: neither the
- * result nor the work depends on the order of dirs (neighbouring rays share cached boxes).
+ * validation is reported as DGS_ERR_INVALID_ARG).  Rays are traced by themselves; in calls of 65,536
+ * rays or more, beams (s, j) .. (s, j + 31) that lie within about half a degree of one direction are
+ * traced together as a packet, so order dense patterns such that every 32 consecutive directions are
+ * neighbours (e.g. tiles of 4 channels x 8 azimuths).  The result does not depend on the order.
  */
 int dgs_lidar_trace(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nodes,
                     const int32_t* env_node_ids, int32_t n_envs, int32_t max_nodes, const float* node_poses,

@@ -2007,7 +2007,9 @@ int dgs_lidar_trace(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nodes, const 
     const size_t o_slot = align_up(sizeof(LidarSensorDev) * n_sensors, 256);
     const size_t bytes = o_slot + sizeof(int32_t) * (size_t)E * K;
     if ((rc = ensure(ctx, ctx->lid_meta, bytes))) return rc;
-    if ((rc = ensure(ctx, ctx->lid_slots, sizeof(LidarSlot) * (size_t)n_sensors * K))) return rc;
+    const int64_t n_rays = (int64_t)n_sensors * n_dirs;
+    const size_t o_packets = align_up(sizeof(LidarSlot) * (size_t)n_sensors * K, 256);
+    if ((rc = ensure(ctx, ctx->lid_slots, o_packets + sizeof(uint32_t) * lidar_packet_words(n_rays)))) return rc;
     if ((rc = ensure(ctx, ctx->errword, 64))) return rc;
     if ((rc = ensure_host(ctx, ctx->h_lid, ctx->h_lid_bytes, bytes))) return rc;
     DGS_CUDA(ctx, cudaStreamSynchronize(stream));   // the previous call's upload from the staging
@@ -2022,12 +2024,15 @@ int dgs_lidar_trace(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nodes, const 
     Timer tm{ctx, stream, ctx->opt.profile != 0};
     tm.begin(DGS_K_LIDAR);
     LidarSlot* slots = static_cast<LidarSlot*>(ctx->lid_slots.p);
+    const LidarPackets packets = lidar_packets(
+        n_rays, reinterpret_cast<uint32_t*>(static_cast<char*>(ctx->lid_slots.p) + o_packets), err + 4);
     launch_lidar_setup(L, reinterpret_cast<const LidarSensorDev*>(d), n_sensors,
-                       reinterpret_cast<const int32_t*>(d + o_slot), K, node_poses, slots, err);
+                       reinterpret_cast<const int32_t*>(d + o_slot), K, node_poses, slots, err, dirs, n_dirs, n_rays,
+                       packets);
     LidarParams LP{r_min, r_max, ctx->opt.alpha_min, ctx->opt.alpha_max, ctx->opt.t_min, ctx->opt.q_max};
     launch_lidar_trace(L, static_cast<const LidarTreeDev*>(ctx->lid_tab.p), slots, K, dirs, n_dirs,
-                       (int64_t)n_sensors * n_dirs, LP, out_d, out_a, err,
-                       reinterpret_cast<unsigned long long*>(static_cast<char*>(ctx->errword.p) + 8));
+                       n_rays, LP, out_d, out_a, err,
+                       reinterpret_cast<unsigned long long*>(err + 2), packets);
     tm.end();
     DGS_CUDA(ctx, cudaGetLastError());
     uint32_t errw = 0;

@@ -661,16 +661,27 @@ struct LidarSlot {           // per (sensor, slot): sensor in the node's frame
 struct LidarParams {
     float r_min, r_max, alpha_min, alpha_max, t_min, q_max;
 };
+// Packets of 32 consecutive rays (n = 0: none are looked for).
+struct LidarPackets {
+    uint32_t n;
+    float cone;                          // radius in radians of the directions of a packet traced together
+    uint32_t *together, *left;           // packets traced together, and those whose rays are traced one by one
+    uint32_t *next, *counts;             // the next packet to take; the lists' lengths
+};
+// scratch: lidar_packet_words(n_rays) words; counters: three words, zero on entry.
+size_t lidar_packet_words(int64_t n_rays);
+LidarPackets lidar_packets(int64_t n_rays, uint32_t* scratch, uint32_t* counters);
 size_t lidar_tree_nodes(int64_t n);
 void launch_lidar_records(const Launch& L, const NodeDesc& nd, float q_max, float4* rec, float4* box, int64_t P);
 size_t lidar_level_job_bytes();
 void lidar_level_job(void* jobs, int i, float4* box, int64_t first);
 void launch_lidar_level(const Launch& L, const void* jobs, int n_jobs, int64_t h, int64_t total);
 void launch_lidar_setup(const Launch& L, const LidarSensorDev* sensors, int S, const int32_t* slot_node, int K,
-                        const float* node_poses, LidarSlot* out, uint32_t* err);
+                        const float* node_poses, LidarSlot* out, uint32_t* err, const float* dirs, int n_dirs,
+                        int64_t n_rays, const LidarPackets& packets);
 void launch_lidar_trace(const Launch& L, const LidarTreeDev* trees, const LidarSlot* slots, int K, const float* dirs,
                         int n_dirs, int64_t n_rays, const LidarParams& LP, float* out_d, float* out_a, uint32_t* err,
-                        unsigned long long* next_ray);
+                        unsigned long long* next_ray, const LidarPackets& packets);
 
 // Mesh -> Gaussian transfer (csrc/mesh.cu): one Gaussian per facet into node-layout arrays
 // (quat must be 16-byte aligned).

@@ -15,8 +15,8 @@
 // tree's quality follows the storage order: Z-ordered nodes (dgs_spatial_order) give compact
 // leaves.  Trees are never refitted per env: rays are moved into each node's frame instead.
 //
-// Tracing: one warp per ray, its lanes testing 32 boxes or 32 Gaussians at a time (see
-// k_lidar_trace).
+// Tracing: one warp per ray, its lanes testing 32 boxes or 32 Gaussians at a time (k_lidar_trace); in
+// dense beam patterns one warp per packet of 32 neighbouring rays (k_lidar_packets).
 #include <algorithm>
 
 #include "dgs_internal.cuh"
@@ -107,10 +107,64 @@ __global__ void k_lidar_level(const LevelJob* __restrict__ jobs, int n_jobs, int
     box[2 * k + 1] = make_float4(fmaxf(a1.x, b1.x), fmaxf(a1.y, b1.y), fmaxf(a1.z, b1.z), 0.f);
 }
 
-// Per (sensor, slot): the sensor's rotation and origin expressed in the node's frame.
-__global__ void k_lidar_setup(const LidarSensorDev* __restrict__ sensors, int S, const int32_t* __restrict__ slot_node,
-                              int K, const float* __restrict__ node_poses, LidarSlot* __restrict__ out,
-                              uint32_t* __restrict__ err) {
+// A sensor's beam j: its unit direction.
+__device__ __forceinline__ void sensor_ray(const float* __restrict__ dirs, int64_t j, float (&ds)[3]) {
+    ds[0] = dirs[3 * j]; ds[1] = dirs[3 * j + 1]; ds[2] = dirs[3 * j + 2];
+    const float r = rsqrtf(ds[0] * ds[0] + ds[1] * ds[1] + ds[2] * ds[2]);
+    ds[0] *= r; ds[1] *= r; ds[2] *= r;
+}
+
+// The packets of 32 rays, one per warp of the block: those whose directions lie within `cone` of their mean
+// are listed to be traced together (k_lidar_packets), the others to be left to k_lidar_trace; counts =
+// their numbers, to which a block adds once.
+__device__ __forceinline__ void list_packets(uint32_t block, const float* __restrict__ dirs, int n_dirs,
+                                             int64_t n_rays, const LidarPackets& L) {
+    __shared__ uint32_t s_near[32], s_first[2];
+    const uint32_t lane = lane_id(), warp = threadIdx.x >> 5, full = 0xffffffffu;
+    const int64_t ray0 = ((int64_t)block * 32 + warp) * 32, j0 = ray0 % n_dirs;
+    bool near = ray0 + 32 <= n_rays && j0 + 32 <= n_dirs;            // 32 rays of one sensor
+    if (near) {
+        float ds[3], m[3];
+        sensor_ray(dirs, j0 + lane, ds);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            m[a] = ds[a];
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) m[a] += __shfl_xor_sync(full, m[a], o);
+        }
+        const float r = rsqrtf(m[0] * m[0] + m[1] * m[1] + m[2] * m[2]);
+        const float e0 = ds[0] - m[0] * r, e1 = ds[1] - m[1] * r, e2 = ds[2] - m[2] * r;
+        near = __all_sync(full, fmaf(e0, e0, fmaf(e1, e1, e2 * e2)) <= L.cone * L.cone);
+    }
+    if (lane == 0) s_near[warp] = near;
+    __syncthreads();
+    if (warp != 0) return;
+    const uint32_t pk = block * 32u + lane;
+    const bool in = pk < L.n && s_near[lane], out = pk < L.n && !in;
+    const uint32_t m_in = __ballot_sync(full, in), m_out = __ballot_sync(full, out);
+    if (lane < 2) {
+        const uint32_t n = __popc(lane ? m_out : m_in);
+        s_first[lane] = n ? atomicAdd(L.counts + lane, n) : 0u;
+    }
+    __syncwarp();
+    const uint32_t below = (1u << lane) - 1u;
+    if (in) L.together[s_first[0] + __popc(m_in & below)] = pk;
+    if (out) L.left[s_first[1] + __popc(m_out & below)] = pk;
+}
+
+// Per (sensor, slot): the sensor's rotation and origin expressed in the node's frame.  The blocks from
+// setup_blocks on list the packets.
+constexpr int kSetupThreads = 1024;
+__global__ void __launch_bounds__(kSetupThreads) k_lidar_setup(const LidarSensorDev* __restrict__ sensors, int S,
+                                                               const int32_t* __restrict__ slot_node, int K,
+                                                               const float* __restrict__ node_poses,
+                                                               LidarSlot* __restrict__ out, uint32_t* __restrict__ err,
+                                                               unsigned setup_blocks, const float* __restrict__ dirs,
+                                                               int n_dirs, int64_t n_rays, LidarPackets packets) {
+    if (blockIdx.x >= setup_blocks) {
+        list_packets(blockIdx.x - setup_blocks, dirs, n_dirs, n_rays, packets);
+        return;
+    }
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= S * K) return;
     const int s = idx / K, j = idx % K;
@@ -193,6 +247,33 @@ __device__ __forceinline__ NodeRay node_ray(const LidarSlot& S, const float (&ds
         r.id[a] = 1.f / r.d[a];
     }
     return r;
+}
+
+// A ray against the Gaussian of record (r0, r1, r2, r3): whether its peak lies within q_max and the
+// range window, with its distance t and Mahalanobis distance q.
+__device__ __forceinline__ bool peak(const float4 r0, const float4 r1, const float4 r2, const float4 r3, const NodeRay& R,
+                                     const LidarParams& LP, float& t, float& q) {
+    const float v0 = R.o[0] - r0.x, v1 = R.o[1] - r0.y, v2 = R.o[2] - r0.z;
+    const float x0 = fmaf(v1, R.d[2], -v2 * R.d[1]), x1 = fmaf(v2, R.d[0], -v0 * R.d[2]),
+                x2 = fmaf(v0, R.d[1], -v1 * R.d[0]);
+    if (fmaf(x0, x0, fmaf(x1, x1, x2 * x2)) > r3.y) return false;   // |d| = 1 up to rounding
+    const float op0 = fmaf(r1.x, v0, fmaf(r1.y, v1, r1.z * v2));
+    const float op1 = fmaf(r1.w, v0, fmaf(r2.x, v1, r2.y * v2));
+    const float op2 = fmaf(r2.z, v0, fmaf(r2.w, v1, r3.x * v2));
+    const float dp0 = fmaf(r1.x, R.d[0], fmaf(r1.y, R.d[1], r1.z * R.d[2]));
+    const float dp1 = fmaf(r1.w, R.d[0], fmaf(r2.x, R.d[1], r2.y * R.d[2]));
+    const float dp2 = fmaf(r2.z, R.d[0], fmaf(r2.w, R.d[1], r3.x * R.d[2]));
+    const float dd = fmaf(dp0, dp0, fmaf(dp1, dp1, dp2 * dp2));
+    const float od = fmaf(op0, dp0, fmaf(op1, dp1, op2 * dp2));
+    const float c0 = fmaf(op1, dp2, -op2 * dp1), c1 = fmaf(op2, dp0, -op0 * dp2), c2 = fmaf(op0, dp1, -op1 * dp0);
+    const float idd = 1.f / dd;
+    t = -od * idd;
+    q = fmaf(c0, c0, fmaf(c1, c1, c2 * c2)) * idd;
+    return q <= LP.q_max && t >= LP.r_min && t <= LP.r_max;
+}
+
+__device__ __forceinline__ float hit_alpha(float opacity, float q, const LidarParams& LP) {
+    return fminf(LP.alpha_max, opacity * fast_exp2(kHalfLog2e * q));
 }
 
 // Pushes the lanes with `in` set onto the stack, nearest entry on top (ties by lane).
@@ -295,6 +376,12 @@ __device__ __forceinline__ uint64_t cut_pending(RayWarp& W, int& cnt, int lane) 
     return x;
 }
 
+// Whether the packets listed as together (counts[0]) are traced so: half of all at least.  Fewer leave
+// both kernels too little to do, one after the other.
+__device__ __forceinline__ bool packets_taken(const uint32_t* counts, int64_t n_rays) {
+    return 64ll * counts[0] >= n_rays;
+}
+
 // Warp = one ray at a time; persistent warps take the next ray from a counter.  Beams of a
 // sensor are farther apart, at the distances where they hit, than the Gaussians are wide, so
 // neighbouring rays share few leaves: the 32 lanes work on one ray instead, 32 boxes or 32
@@ -313,33 +400,37 @@ __device__ __forceinline__ uint64_t cut_pending(RayWarp& W, int& cnt, int lane) 
 // hits beyond them are skipped, and another round resumes after them.  The trees of up to 32
 // slots share one stack; with more, a slot batch is traversed after the other and hits are
 // final at the end of the round only.
-// Bound by latency (boxes and records come from L2, one dependent load per step) and at 66 % issue;
-// 64 registers keep 32 warps an SM.  Same outputs bit for bit, one sensor of 32 x 1024 beams through
-// 380k Gaussians and 16 sensors through 580k: a packet of 32 rays per warp with a 32-hit buffer per
-// lane 7.4 and 28 ms (with one sensor the slowest packet was the time); one ray per warp, one node
-// of five levels per expansion, 72 registers 0.592 and 5.59 ms; two nodes 0.588 and 5.51; with 64
-// registers 0.555 and 5.04.
+// Bound by latency (boxes and records come from L2, one dependent load per step); 64 registers keep 32
+// warps an SM.  Same outputs bit for bit: one sensor of 32 x 1024 beams through 380k Gaussians and 16
+// sensors through 580k took 9-15 and 20-33 ms (by scene) with a packet of 32 rays per warp, where the
+// slowest packet is the time; one ray per warp, one node of five levels per expansion, 72 registers
+// 0.592 and 5.59 ms; two nodes 0.588 and 5.51; with 64 registers 0.555 and 5.04.
+//
+// LISTED: the rays are those of the packets that are not traced together, or that k_lidar_packets left.
+template <bool LISTED>
 __global__ void __launch_bounds__(kRayWarps * 32, 8) k_lidar_trace(const LidarTreeDev* __restrict__ trees,
                                                                 const LidarSlot* __restrict__ slots, int K,
                                                                 const float* __restrict__ dirs, int n_dirs,
                                                                 int64_t n_rays, LidarParams LP,
                                                                 float* __restrict__ out_d, float* __restrict__ out_a,
                                                                 uint32_t* __restrict__ err,
-                                                                unsigned long long* __restrict__ next_ray) {
+                                                                unsigned long long* __restrict__ next_ray,
+                                                                const uint32_t* __restrict__ left,
+                                                                const uint32_t* __restrict__ counts) {
     __shared__ RayWarp s_warp[kRayWarps];
     const int lane = threadIdx.x & 31;
     RayWarp& W = s_warp[threadIdx.x >> 5];
+    const bool some = LISTED && packets_taken(counts, n_rays);   // (else all rays, in order)
     for (;;) {
         unsigned long long ray = 0;
         if (lane == 0) ray = atomicAdd(next_ray, 1ull);
         ray = __shfl_sync(0xffffffffu, ray, 0);
-        if (ray >= (unsigned long long)n_rays) break;
+        if (ray >= (some ? 32ull * __ldg(counts + 1) : (unsigned long long)n_rays)) break;
+        if (some) ray = 32ull * left[ray >> 5] + (ray & 31ull);
+        if (some && ray >= (unsigned long long)n_rays) continue;
         const int64_t s = (int64_t)ray / n_dirs, j = (int64_t)ray - s * n_dirs;
-        float ds[3] = {dirs[3 * j], dirs[3 * j + 1], dirs[3 * j + 2]};
-        {
-            const float r = rsqrtf(ds[0] * ds[0] + ds[1] * ds[1] + ds[2] * ds[2]);
-            ds[0] *= r; ds[1] *= r; ds[2] *= r;
-        }
+        float ds[3];
+        sensor_ray(dirs, j, ds);
         const LidarSlot* sl = slots + s * K;
         float T = 1.f, D = 0.f;
         uint64_t last = 0;                             // keys <= last are composited
@@ -424,29 +515,12 @@ __global__ void __launch_bounds__(kRayWarps * 32, 8) k_lidar_trace(const LidarTr
                 if (g >= 0 && g < tr.n) {
                     const float4* rp = tr.rec + 4 * g;
                     const float4 r0 = __ldg(rp), r1 = __ldg(rp + 1), r2 = __ldg(rp + 2), r3 = __ldg(rp + 3);
-                    const float v0 = R.o[0] - r0.x, v1 = R.o[1] - r0.y, v2 = R.o[2] - r0.z;
-                    const float x0 = fmaf(v1, R.d[2], -v2 * R.d[1]), x1 = fmaf(v2, R.d[0], -v0 * R.d[2]),
-                                x2 = fmaf(v0, R.d[1], -v1 * R.d[0]);
-                    if (!(fmaf(x0, x0, fmaf(x1, x1, x2 * x2)) > r3.y)) {   // |d| = 1 up to rounding
-                        const float op0 = fmaf(r1.x, v0, fmaf(r1.y, v1, r1.z * v2));
-                        const float op1 = fmaf(r1.w, v0, fmaf(r2.x, v1, r2.y * v2));
-                        const float op2 = fmaf(r2.z, v0, fmaf(r2.w, v1, r3.x * v2));
-                        const float dp0 = fmaf(r1.x, R.d[0], fmaf(r1.y, R.d[1], r1.z * R.d[2]));
-                        const float dp1 = fmaf(r1.w, R.d[0], fmaf(r2.x, R.d[1], r2.y * R.d[2]));
-                        const float dp2 = fmaf(r2.z, R.d[0], fmaf(r2.w, R.d[1], r3.x * R.d[2]));
-                        const float dd = fmaf(dp0, dp0, fmaf(dp1, dp1, dp2 * dp2));
-                        const float od = fmaf(op0, dp0, fmaf(op1, dp1, op2 * dp2));
-                        const float c0 = fmaf(op1, dp2, -op2 * dp1), c1 = fmaf(op2, dp0, -op0 * dp2),
-                                    c2 = fmaf(op0, dp1, -op1 * dp0);
-                        const float idd = 1.f / dd;
-                        t = -od * idd;
-                        const float q = fmaf(c0, c0, fmaf(c1, c1, c2 * c2)) * idd;
-                        if (q <= LP.q_max && t >= LP.r_min && t <= LP.r_max) {
-                            const uint64_t key = ((uint64_t)__float_as_uint(t) << 32) | (uint32_t)(tr.gbase + g);
-                            if ((first || key > last) && key < maxkey) {
-                                alpha = fminf(LP.alpha_max, r0.w * fast_exp2(kHalfLog2e * q));
-                                hit = alpha >= LP.alpha_min;
-                            }
+                    float q;
+                    if (peak(r0, r1, r2, r3, R, LP, t, q)) {
+                        const uint64_t key = ((uint64_t)__float_as_uint(t) << 32) | (uint32_t)(tr.gbase + g);
+                        if ((first || key > last) && key < maxkey) {
+                            alpha = hit_alpha(r0.w, q, LP);
+                            hit = alpha >= LP.alpha_min;
                         }
                     }
                 }
@@ -489,6 +563,168 @@ __global__ void __launch_bounds__(kRayWarps * 32, 8) k_lidar_trace(const LidarTr
     }
 }
 
+// The packets listed as together, 32 neighbouring rays of one sensor each: warp = packet, lane = ray.  The
+// packet walks each tree together on a warp-uniform stack: a box is descended if any lane's interval meets
+// it, the children in the order of the first such lane's entries; boxes and records are read once for
+// the packet.  A lane keeps the kHits nearest hits of a round, sorted, in shared memory; a round's hits
+// are composited in order and the next resumes after the last of them, until every lane's
+// transmittance has ended or its hits have run out.  A packet that takes too many nodes (rays grazing a
+// surface, an object's dense centre: up to 10 ms for one packet) is left to k_lidar_trace, which
+// finds the same hits.
+//
+// Rays so close that they meet the same leaves cost k_lidar_trace 32 walks of them, 5 ns a ray with the
+// chip full; a packet walks the union once.  Bound by latency (16 warps an SM, one dependent load per
+// step), so packets pay where there are enough of them and their cones are narrow.  Whole calls, 300k
+// Gaussians of a room, against k_lidar_trace alone: 1024 x 1024 beams over 5 x 2.5 degrees 5.10 -> 1.22 ms,
+// over 160 x 80 6.89 -> 2.66; 512 x 512 over 20 x 10 1.50 -> 0.53, over 80 x 40 2.06 -> 1.40 (with four
+// objects of 20k beside it 2.88 -> 3.00); 256 x 256 over 10 x 5 0.41 -> 0.21.  Not taken, for what they would
+// take: 64 x 1024 over 360 x 41 degrees 0.52 against 1.23, 512 x 512 over 160 x 80 1.79 against 1.39 (with
+// the objects 2.28 against 2.77).  Budgets of 512 and 2048 nodes: 1.67 and 1.28 ms for 512 x 512 over
+// 80 x 40, 2.87 and 4.25 with the objects.
+constexpr int kPacketThreads = 128;
+constexpr int kHits = 32;
+constexpr int kWalk = 64;            // a level's sibling on the stack at most: 29
+constexpr int kPacketSteps = 1024;   // nodes a packet may take before its rays are left
+constexpr size_t kPacketSmem = (size_t)3 * kHits * kPacketThreads * sizeof(uint32_t);   // [entry][thread]: t bits, id, alpha
+
+__global__ void __launch_bounds__(kPacketThreads, 4) k_lidar_packets(const LidarTreeDev* __restrict__ trees,
+                                                                  const LidarSlot* __restrict__ slots, int K,
+                                                                  const float* __restrict__ dirs, int n_dirs,
+                                                                  int64_t n_rays, LidarParams LP,
+                                                                  float* __restrict__ out_d,
+                                                                  float* __restrict__ out_a, uint32_t* __restrict__ err,
+                                                                  LidarPackets packets) {
+    __shared__ uint32_t s_stack[kPacketThreads / 32][kWalk];
+    extern __shared__ uint32_t s_hits[];
+    uint32_t* const kt = s_hits + threadIdx.x;                      // entry i at kt[i * kPacketThreads]
+    uint32_t* const kg = kt + kHits * kPacketThreads;
+    float* const ka = reinterpret_cast<float*>(kg + kHits * kPacketThreads);
+    const int lane = threadIdx.x & 31;
+    const unsigned full = 0xffffffffu;
+    uint32_t* const stk = s_stack[threadIdx.x >> 5];
+    if (!packets_taken(packets.counts, n_rays)) return;
+    for (;;) {
+        uint32_t at = 0;
+        if (lane == 0) at = atomicAdd(packets.next, 1u);
+        at = __shfl_sync(full, at, 0);
+        if (at >= packets.counts[0]) break;
+        const uint32_t pk = packets.together[at];
+        const int64_t ray0 = (int64_t)pk * 32, s = ray0 / n_dirs;
+        float ds[3];
+        sensor_ray(dirs, ray0 - s * n_dirs + lane, ds);
+        int steps = 0;                                 // nodes taken from the stack
+        const LidarSlot* sl = slots + s * K;
+        float T = 1.f, D = 0.f;
+        uint64_t last = 0;                             // keys <= last are composited
+        bool first = true, done = false;
+        while (__any_sync(full, !done) && steps <= kPacketSteps) {   // a round
+            int cnt = 0;
+            uint64_t maxkey = ~0ull;                   // key of the last entry once the buffer is full
+            const float t_lo = first ? LP.r_min : __uint_as_float((uint32_t)(last >> 32));
+            float t_hi = LP.r_max;
+            for (int slot = 0; slot < K; ++slot) {
+                const LidarSlot& S = sl[slot];
+                if (S.node < 0) continue;
+                const LidarTreeDev tr = trees[S.node];
+                if (tr.n == 0) continue;
+                const NodeRay R = node_ray(S, ds);
+                int sp = 0;
+                if (__any_sync(full, !done && slab(tr.box[2], tr.box[3], R.o, R.id, t_lo, t_hi))) {
+                    if (lane == 0) stk[0] = 1u;
+                    sp = 1;
+                }
+                __syncwarp();
+                while (sp > 0 && ++steps <= kPacketSteps) {
+                    const uint32_t k = stk[--sp];
+                    __syncwarp();                      // every lane has read before lane 0 writes
+                    if ((int64_t)k < tr.P) {
+                        const float4* b = tr.box + 4 * (size_t)k;      // the children 2k and 2k + 1
+                        const float4 l0 = __ldg(b), h0 = __ldg(b + 1), l1 = __ldg(b + 2), h1 = __ldg(b + 3);
+                        const unsigned b0 = __ballot_sync(full, !done && slab(l0, h0, R.o, R.id, t_lo, t_hi));
+                        const unsigned b1 = __ballot_sync(full, !done && slab(l1, h1, R.o, R.id, t_lo, t_hi));
+                        if (!(b0 | b1)) continue;
+                        const int more = b0 && b1 ? 2 : 1;
+                        bool zero = b0 != 0;
+                        if (more == 2) {
+                            const bool near0 = slab_enter(l0, h0, R.o, R.id) <= slab_enter(l1, h1, R.o, R.id);
+                            zero = __shfl_sync(full, near0, __ffs(b0 | b1) - 1);
+                        }
+                        if (sp + more > kWalk) {       // cannot happen for trees of the documented sizes
+                            if (lane == 0) atomicOr(err, kErrCapacity);
+                            break;
+                        }
+                        if (lane == 0) {               // far child below, near on top
+                            if (more == 2) stk[sp] = 2u * k + (zero ? 1u : 0u);
+                            stk[sp + more - 1] = 2u * k + (zero ? 0u : 1u);
+                        }
+                        sp += more;
+                        __syncwarp();
+                        continue;
+                    }
+                    const int64_t g0 = ((int64_t)k - tr.P) * kLeaf, g1 = min(g0 + kLeaf, tr.n);
+                    // the next Gaussian's record is loaded while this one is tested
+                    float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0, n2 = n0, n3 = n0;
+                    auto load = [&](int64_t g) {
+                        const float4* rp = tr.rec + 4 * g;
+                        n0 = __ldg(rp); n1 = __ldg(rp + 1); n2 = __ldg(rp + 2); n3 = __ldg(rp + 3);
+                    };
+                    if (g0 < g1) load(g0);
+                    for (int64_t g = g0; g < g1; ++g) {
+                        const float4 r0 = n0, r1 = n1, r2 = n2, r3 = n3;
+                        if (g + 1 < g1) load(g + 1);
+                        float t, q;
+                        if (done || !peak(r0, r1, r2, r3, R, LP, t, q)) continue;
+                        const uint64_t key = ((uint64_t)__float_as_uint(t) << 32) | (uint32_t)(tr.gbase + g);
+                        if ((!first && key <= last) || key >= maxkey) continue;
+                        const float alpha = hit_alpha(r0.w, q, LP);
+                        if (alpha < LP.alpha_min) continue;
+                        // insert in order; a full buffer drops its last entry
+                        int i = min(cnt, kHits - 1);
+                        for (; i > 0; --i) {
+                            const uint32_t pt = kt[(i - 1) * kPacketThreads], pg = kg[(i - 1) * kPacketThreads];
+                            if ((((uint64_t)pt << 32) | pg) < key) break;
+                            kt[i * kPacketThreads] = pt;
+                            kg[i * kPacketThreads] = pg;
+                            ka[i * kPacketThreads] = ka[(i - 1) * kPacketThreads];
+                        }
+                        kt[i * kPacketThreads] = (uint32_t)(key >> 32);
+                        kg[i * kPacketThreads] = (uint32_t)key;
+                        ka[i * kPacketThreads] = alpha;
+                        cnt = min(cnt + 1, kHits);
+                        if (cnt == kHits) {
+                            const uint32_t lt = kt[(kHits - 1) * kPacketThreads];
+                            maxkey = ((uint64_t)lt << 32) | kg[(kHits - 1) * kPacketThreads];
+                            t_hi = __uint_as_float(lt);
+                        }
+                    }
+                    __syncwarp();
+                }
+                __syncwarp();
+            }
+            if (!done) {
+                for (int i = 0; i < cnt && !done; ++i) {
+                    const float a = ka[i * kPacketThreads], Tn = fmaf(-a, T, T);
+                    if (Tn < LP.t_min) {
+                        done = true;
+                    } else {
+                        D = fmaf(a * T, __uint_as_float(kt[i * kPacketThreads]), D);
+                        T = Tn;
+                    }
+                }
+                done |= cnt < kHits;
+                last = maxkey;
+                first = false;
+            }
+        }
+        if (steps > kPacketSteps) {                          // given up: its rays one by one
+            if (lane == 0) packets.left[atomicAdd(packets.counts + 1, 1u)] = pk;
+            continue;
+        }
+        out_d[ray0 + lane] = D;
+        out_a[ray0 + lane] = 1.f - T;
+    }
+}
+
 }  // namespace
 
 size_t lidar_tree_nodes(int64_t n) {
@@ -525,30 +761,65 @@ void lidar_level_job(void* jobs, int i, float4* box, int64_t first) {
     static_cast<LevelJob*>(jobs)[i] = LevelJob{box, first};
 }
 
+// Rays from which packets are looked for: with fewer, the slowest packet is longer than all rays one by one,
+// but for beams a tenth of a degree apart or less.  The cone widens with the number of packets, which
+// hides the slow ones.
+constexpr int64_t kPacketRays = 1 << 16;
+constexpr float kPacketCone = 0.010471976f;             // 0.6 degrees, from
+constexpr int64_t kPacketConeRays = 1 << 17;            // this many rays on, in proportion below
+
+size_t lidar_packet_words(int64_t n_rays) { return n_rays >= kPacketRays ? 2 * (size_t)((n_rays + 31) / 32) : 0; }
+
+LidarPackets lidar_packets(int64_t n_rays, uint32_t* scratch, uint32_t* counters) {
+    LidarPackets p{};
+    p.n = (uint32_t)(lidar_packet_words(n_rays) / 2);
+    p.cone = kPacketCone * std::min(1.f, (float)n_rays / (float)kPacketConeRays);
+    p.together = scratch;
+    p.left = scratch + p.n;
+    p.next = counters;
+    p.counts = counters + 1;
+    return p;
+}
+
 void launch_lidar_setup(const Launch& L, const LidarSensorDev* sensors, int S, const int32_t* slot_node, int K,
-                        const float* node_poses, LidarSlot* out, uint32_t* err) {
+                        const float* node_poses, LidarSlot* out, uint32_t* err, const float* dirs, int n_dirs,
+                        int64_t n_rays, const LidarPackets& packets) {
     const int n = S * K;
     if (n == 0) return;
-    k_lidar_setup<<<(n + 127) / 128, 128, 0, L.stream>>>(sensors, S, slot_node, K, node_poses, out, err);
+    const int threads = packets.n ? kSetupThreads : 128;
+    const unsigned blocks = (unsigned)((n + threads - 1) / threads);
+    k_lidar_setup<<<blocks + (packets.n + 31) / 32, threads, 0, L.stream>>>(sensors, S, slot_node, K, node_poses, out, err,
+                                                                           blocks, dirs, n_dirs, n_rays, packets);
     ++*L.launches;
+}
+
+template <class Kernel>
+static unsigned resident_blocks(Kernel* k, int threads, size_t smem) {
+    int dev = 0, sms = 0, r = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (smem) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, k, threads, smem);
+    return (unsigned)(std::max(r, 1) * sms);
 }
 
 void launch_lidar_trace(const Launch& L, const LidarTreeDev* trees, const LidarSlot* slots, int K, const float* dirs,
                         int n_dirs, int64_t n_rays, const LidarParams& LP, float* out_d, float* out_a, uint32_t* err,
-                        unsigned long long* next_ray) {
+                        unsigned long long* next_ray, const LidarPackets& packets) {
     if (n_rays <= 0) return;
-    static int resident = 0, sms = 0;           // blocks per SM at this kernel's resources
-    if (!resident) {
-        int dev = 0, r = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, k_lidar_trace, kRayWarps * 32, 0);
-        resident = std::max(r, 1);
+    if (packets.n) {
+        static const unsigned most = resident_blocks(k_lidar_packets, kPacketThreads, kPacketSmem);
+        const unsigned need = (packets.n + kPacketThreads / 32 - 1) / (kPacketThreads / 32);
+        k_lidar_packets<<<std::min(need, most), kPacketThreads, kPacketSmem, L.stream>>>(
+            trees, slots, K, dirs, n_dirs, n_rays, LP, out_d, out_a, err, packets);
+        ++*L.launches;
     }
-    const int64_t need = (n_rays + kRayWarps - 1) / kRayWarps;
-    const unsigned blocks = (unsigned)std::min<int64_t>(need, (int64_t)resident * sms);
-    k_lidar_trace<<<blocks, kRayWarps * 32, 0, L.stream>>>(trees, slots, K, dirs, n_dirs, n_rays, LP, out_d, out_a, err,
-                                                           next_ray);
+    auto* kern = packets.n ? k_lidar_trace<true> : k_lidar_trace<false>;
+    static const unsigned most = std::min(resident_blocks(k_lidar_trace<true>, kRayWarps * 32, 0),
+                                          resident_blocks(k_lidar_trace<false>, kRayWarps * 32, 0));
+    const unsigned blocks = (unsigned)std::min<int64_t>((n_rays + kRayWarps - 1) / kRayWarps, most);
+    kern<<<blocks, kRayWarps * 32, 0, L.stream>>>(trees, slots, K, dirs, n_dirs, n_rays, LP, out_d, out_a, err, next_ray,
+                                                  packets.left, packets.counts);
     ++*L.launches;
 }
 
