@@ -106,8 +106,8 @@ typedef struct dgs_options {
                                    streams, one group's binning overlapping the other's compositing;
                                    more groups only where the 2^30-pair or the 2^24-tile limit of a
                                    group needs them */
-    int32_t spin_limit_us;      /* limit of every bounded device-side wait (the sort's look-back), in
-                                   microseconds, 0 = 1 s; a wait that runs out ends the call with
+    int32_t spin_limit_us;      /* limit of every bounded device-side wait (the scans' and the sorts'
+                                   look-back), in microseconds, 0 = 1 s; a wait that runs out ends the call with
                                    DGS_ERR_TIMEOUT (outputs invalid, the context stays usable) */
     int32_t check_binning;      /* 1 = eager renders read each view group's tile lists back and check
                                    them on the host before compositing: tiles non-decreasing and below
@@ -115,10 +115,12 @@ typedef struct dgs_options {
                                    covering every pair once, and each tile's run in depth order (equal
                                    depths by instance number); a violation ends the call with
                                    DGS_ERR_CUDA and a description.  Slow: for tests and debugging */
-    int32_t test_fault;         /* fault injection for tests, 0 = none.  1: the first digit pass of the
-                                   depth sort leaves the look-back status of its second partition
-                                   unpublished, so the waits behind it run out (DGS_ERR_TIMEOUT after
-                                   about spin_limit_us per wave of resident blocks); 2: with
+    int32_t test_fault;         /* fault injection for tests, 0 = none.  1: the scan of the count table
+                                   and the first digit pass of the depth sort leave the look-back
+                                   status of their second partition (of 4096 entries, of 3072
+                                   instances) unpublished, so the waits of those behind it run out
+                                   (DGS_ERR_TIMEOUT after about spin_limit_us per wave of resident
+                                   blocks); 2: with
                                    check_binning, the host copy of the first view group's tile keys is
                                    corrupted (two adjacent pairs of different tiles exchanged) before
                                    the check, which must then report it; 3 (DGS_DEBUG builds only,

@@ -655,11 +655,6 @@ int stage(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nodes, const int32_t* e
     return DGS_OK;
 }
 
-// Limit of the bounded device waits.
-uint64_t spin_limit_ns(const dgs_options& o) {
-    return o.spin_limit_us > 0 ? (uint64_t)o.spin_limit_us * 1000ull : SortCtl{}.spin_ns;
-}
-
 // Clears the error word, then setup (K0), count (K1) and the exclusive scan of the count table.
 void launch_front(dgs_ctx* ctx, const Batch& B, const Launch& L, Timer& tm) {
     cudaMemsetAsync(B.d_err, 0, sizeof(uint32_t) * B.call_words, L.stream);
@@ -678,7 +673,8 @@ void launch_front(dgs_ctx* ctx, const Batch& B, const Launch& L, Timer& tm) {
     }
     tm.end();
     tm.begin(DGS_K_SCAN);
-    launch_scan(L, B.d_counts, B.T, B.d_inst_off, B.d_pair_off, B.d_scan, B.d_err, spin_limit_ns(ctx->opt));
+    launch_scan(L, B.d_counts, B.T, B.d_inst_off, B.d_pair_off, B.d_scan, B.d_err, spin_limit_ns(ctx->opt),
+                ctx->opt.test_fault == 1 ? 1u : 0xFFFFFFFFu);
     tm.end();
 }
 
@@ -1102,7 +1098,7 @@ int finish(dgs_ctx* ctx, const Batch& B, cudaStream_t stream) {
         }
     }
     if (errw & kErrBounds) return bounds_failure(ctx, B.d_err);
-    if (errw & kErrTimeout) return fail(ctx, DGS_ERR_TIMEOUT, "a bounded device wait timed out (sort look-back)");
+    if (errw & kErrTimeout) return fail(ctx, DGS_ERR_TIMEOUT, "a bounded device wait timed out (scan or sort look-back)");
     if (errw & kErrMismatch) return fail(ctx, DGS_ERR_CUDA, "internal: count and emit passes disagree");
     if (errw & kErrCapacity) return fail(ctx, DGS_ERR_CUDA, "internal: tile pairs beyond their bound");
     if (errw & kErrPose) return fail(ctx, DGS_ERR_INVALID_ARG, "a node pose is not finite or not rigid");
@@ -1386,7 +1382,7 @@ int render_graph(dgs_ctx* ctx, Batch& B, float* out_rgb, float* out_depth, float
         ctx->stats.key_bits = ctx->gbits;
         if (errw & kErrPose) return fail(ctx, DGS_ERR_INVALID_ARG, "a node pose is not finite or not rigid");
         if (errw & kErrBounds) return bounds_failure(ctx, B.d_err);
-        if (errw & kErrTimeout) return fail(ctx, DGS_ERR_TIMEOUT, "a bounded device wait timed out (sort look-back)");
+        if (errw & kErrTimeout) return fail(ctx, DGS_ERR_TIMEOUT, "a bounded device wait timed out (scan or sort look-back)");
         if (errw & kErrMismatch) return fail(ctx, DGS_ERR_CUDA, "internal: count and emit passes disagree");
         if (!(errw & kErrCapacity) || !sizes[2]) {
             if (errw & kErrCapacity) return fail(ctx, DGS_ERR_CUDA, "internal: tile pairs beyond their bound");

@@ -469,11 +469,11 @@ void launch_count(const Launch& L, int dtype_mask, const NodeDesc* nodes, int n_
 
 // Exclusive scan of the count table: inst_off[n + 1] (32 bits, wrapping), pair_off[n + 1].  scratch:
 // scan_words(n) words, 16-byte aligned and zero on entry; *scan_total(scratch) receives the 64-bit
-// totals (n > 0).
+// totals (n > 0).  mute_part: a partition that publishes no sum (a test of the bounded wait).
 size_t scan_words(int64_t n);
 ulonglong2* scan_total(uint32_t* scratch);
 void launch_scan(const Launch& L, const uint2* counts, int64_t n, uint32_t* inst_off, uint64_t* pair_off,
-                 uint32_t* scratch, uint32_t* err, uint64_t spin_ns);
+                 uint32_t* scratch, uint32_t* err, uint64_t spin_ns, uint32_t mute_part = 0xFFFFFFFFu);
 
 // K2: for every visible instance of views [v0, v1): its record, identity, depth key
 // (bits(z32) - zbase saturated to 28 bits), its own index (the value the depth sort carries)
@@ -483,6 +483,11 @@ void launch_emit(const Launch& L, int dtype_mask, const NodeDesc* nodes, int n_n
                  int n_chunks_total, const Params& P, int v0, int v1, bool batched, const int32_t* view_chunk_nodes,
                  int64_t view_first, int64_t view_chunks, const uint2* counts, const uint32_t* inst_off, uint32_t inst_base,
                  Record* records, InstInfo* info, uint32_t* dkey, uint32_t* ival, uint32_t* ntile, uint32_t* vig);
+
+// Limit of the bounded device waits of a call.
+inline uint64_t spin_limit_ns(const dgs_options& o) {
+    return o.spin_limit_us > 0 ? (uint64_t)o.spin_limit_us * 1000ull : 1000000000ull;
+}
 
 // Bounded waits of the sort: the look-back spin limit, and a test of it (mute_part: the
 // partition of the first digit pass that publishes no status; ~0 = none).

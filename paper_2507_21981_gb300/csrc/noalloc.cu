@@ -154,11 +154,13 @@ extern "C" int dgs_render_noalloc(const dgs_options* opt, const dgs_node* nodes,
     P.err = d_err;
     int64_t launches = 0;
     Launch L{stream, &launches};
+    const uint64_t spin_ns = spin_limit_ns(o);
+    const uint32_t mute = o.test_fault == 1 ? 1u : 0xFFFFFFFFu;
     launch_setup_views(L, d_views, V, node_poses, d_slot, K, d_vnodes, d_err);
     launch_count(L, dtype_mask, d_nodes, n_nodes, d_views, d_vnodes, K, d_nv, d_nvoff, (int)chunk_total, P, 0, V, true,
                  nullptr, 0, 0, d_counts);
     NA_CUDA(cudaMemsetAsync(d_scan, 0, sizeof(uint32_t) * scan_words(T), stream));
-    launch_scan(L, d_counts, T, d_inst_off, d_pair_off, d_scan, d_err, SortCtl{}.spin_ns);
+    launch_scan(L, d_counts, T, d_inst_off, d_pair_off, d_scan, d_err, spin_ns, mute);
     // one view group: read back the grand totals and the error word
     NA_CUDA(cudaMemsetAsync(d_rb, 0, sizeof(uint64_t) * 3, stream));
     // the 64-bit instance total of the scan (its 32-bit offsets wrap beyond 2^32)
@@ -227,6 +229,8 @@ extern "C" int dgs_render_noalloc(const dgs_options* opt, const dgs_node* nodes,
                 nullptr, 0, 0, d_counts, d_inst_off, 0u, d_rec, d_info, d_dk0, d_iv0, d_ntile, vk.vig ? d_vig : nullptr);
     uint32_t *dk, *order, *tk, *tv;
     SortCtl depth_ctl;
+    depth_ctl.spin_ns = spin_ns;
+    depth_ctl.mute_part = mute;
     depth_ctl.runs = true;
     depth_ctl.compact = compact;
     launch_sort(L, d_dk0, d_iv0, d_dk1, d_iv1, (uint32_t)n_vis, plan.depth_bits, d_scratch + plan.depth, d_err,
@@ -235,6 +239,7 @@ extern "C" int dgs_render_noalloc(const dgs_options* opt, const dgs_node* nodes,
                      d_total, d_err, depth_ctl.spin_ns);
     launch_pairs(L, d_views, K, order, d_poff, d_rec, d_info, (uint32_t)n_vis, nullptr, P, d_k0, d_v0, (uint32_t)n_pairs);
     SortCtl tile_ctl;
+    tile_ctl.spin_ns = spin_ns;
     tile_ctl.runs = true;
     tile_ctl.compact = compact;
     if (compact)

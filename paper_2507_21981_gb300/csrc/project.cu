@@ -813,18 +813,20 @@ __device__ __forceinline__ void load_tile_counts(const uint2* __restrict__ count
 }
 
 // Decoupled look-back over 64-bit sums (a 2-bit flag above 62 bits), by one warp: publishes this
-// partition's sum and returns the sum of those before it.  Bounded like the sort's.
+// partition's sum (unless it is muted, a test) and returns the sum of those before it.  Bounded like
+// the sort's.
 constexpr uint64_t kAgg64 = 1ull << 62, kInc64 = 2ull << 62, kSum64 = (1ull << 62) - 1ull;
 
 __device__ __forceinline__ uint64_t look_back64(uint64_t* status, int64_t part, uint64_t sum, int lane, uint32_t* err,
-                                                uint64_t spin_ns) {
+                                                uint64_t spin_ns, bool publish) {
     auto ld = [&](int64_t i) {
         uint64_t v;
         asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(status + i) : "memory");
         return v;
     };
     auto st = [&](uint64_t v) { asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(status + part), "l"(v) : "memory"); };
-    if (lane == 0) st((part == 0 ? kInc64 : kAgg64) | sum);
+    publish &= lane == 0;
+    if (publish) st((part == 0 ? kInc64 : kAgg64) | sum);
     if (part == 0) return 0;
     uint64_t excl = 0, t0 = 0;
     uint32_t spins = 0;
@@ -853,7 +855,7 @@ __device__ __forceinline__ uint64_t look_back64(uint64_t* status, int64_t part, 
             break;
         }
     }
-    if (lane == 0) st(kInc64 | ((excl + sum) & kSum64));
+    if (publish) st(kInc64 | ((excl + sum) & kSum64));
     return excl;
 }
 
@@ -863,7 +865,7 @@ __device__ __forceinline__ uint64_t look_back64(uint64_t* status, int64_t part, 
 // or the graph's size check, stops the call before anything is written through them.
 __global__ void __launch_bounds__(kScanThreads) k_scan(const uint2* __restrict__ counts, int64_t n, uint32_t* counter,
                                                       uint64_t* status, ulonglong2* total, uint32_t* inst_off,
-                                                      uint64_t* pair_off, uint32_t* err, uint64_t spin_ns) {
+                                                      uint64_t* pair_off, uint32_t* err, uint64_t spin_ns, uint32_t mute_part) {
     __shared__ uint2 s_c[kScanPadded];
     __shared__ uint32_t s_part;
     __shared__ uint64_t s_excl[2];
@@ -881,7 +883,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const uint2* __restrict__
     block_excl_scan2(a, b, ta, tb);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (warp < 2) {
-        const uint64_t e = look_back64(status + warp * parts, part, warp ? tb : ta, lane, err, spin_ns);
+        const uint64_t e = look_back64(status + warp * parts, part, warp ? tb : ta, lane, err, spin_ns, part != mute_part);
         if (lane == 0) s_excl[warp] = e;
     }
     __syncthreads();
@@ -1003,7 +1005,7 @@ size_t scan_words(int64_t n) { return 8 + 4 * (size_t)((n + kScanTile - 1) / kSc
 ulonglong2* scan_total(uint32_t* scratch) { return reinterpret_cast<ulonglong2*>(scratch + 4); }
 
 void launch_scan(const Launch& L, const uint2* counts, int64_t n, uint32_t* inst_off, uint64_t* pair_off,
-                 uint32_t* scratch, uint32_t* err, uint64_t spin_ns) {
+                 uint32_t* scratch, uint32_t* err, uint64_t spin_ns, uint32_t mute_part) {
     const int64_t n_parts = (n + kScanTile - 1) / kScanTile;
     if (n_parts == 0) {
         cudaMemsetAsync(inst_off, 0, sizeof(uint32_t), L.stream);
@@ -1011,7 +1013,7 @@ void launch_scan(const Launch& L, const uint2* counts, int64_t n, uint32_t* inst
         return;
     }
     k_scan<<<(unsigned)n_parts, kScanThreads, 0, L.stream>>>(counts, n, scratch, reinterpret_cast<uint64_t*>(scratch + 8),
-                                                             scan_total(scratch), inst_off, pair_off, err, spin_ns);
+                                                             scan_total(scratch), inst_off, pair_off, err, spin_ns, mute_part);
     ++*L.launches;
 }
 
