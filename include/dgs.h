@@ -130,8 +130,9 @@ typedef struct dgs_options {
                                    (DGS_ERR_CUDA naming the check) while every access it lets
                                    through stays inside the records written; 4: not a fault -- the
                                    depth sort takes each instance's view from a separate array even
-                                   where it fits in the instance numbers' high bits (the form of
-                                   view groups too large for that), with identical results */
+                                   where it fits above the depth key (up to 16 views) or in the
+                                   instance numbers' high bits (the form of view groups too large for
+                                   either), with identical results */
     int32_t keep_lists;         /* 1 = a render of at most two view groups -- eager, or a graph
                                    replay (not the call that captures) -- keeps its tile lists,
                                    records and device tables on the context, and a
