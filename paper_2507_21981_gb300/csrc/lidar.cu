@@ -267,7 +267,7 @@ __device__ __forceinline__ bool peak(const float4 r0, const float4 r1, const flo
     const float od = fmaf(op0, dp0, fmaf(op1, dp1, op2 * dp2));
     const float c0 = fmaf(op1, dp2, -op2 * dp1), c1 = fmaf(op2, dp0, -op0 * dp2), c2 = fmaf(op0, dp1, -op1 * dp0);
     const float idd = 1.f / dd;
-    t = -od * idd;
+    t = fmaf(-od, idd, 0.f);           // never -0, whose bits would order it last
     q = fmaf(c0, c0, fmaf(c1, c1, c2 * c2)) * idd;
     return q <= LP.q_max && t >= LP.r_min && t <= LP.r_max;
 }
