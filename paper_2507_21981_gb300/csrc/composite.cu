@@ -445,16 +445,18 @@ void launch_composite(const Launch& L, const ViewDesc* views, int v0, int n_grou
     if (n_tiles == 0) return;
     // checkpoints are for the adjoint, which never runs on randomised outputs
     const bool with_ck = ck.st != nullptr && !P.aug;
-    // few waves: fewer resident blocks with more registers shorten the longest lists' chains;
-    // many waves: the most blocks that fit.  One-group times with 14 against 16 blocks an SM: 64 tiles
-    // 16.4 against 18.4 us, 2400 tiles 71.6 / 80, 19200 tiles 268 / 264, 153600 tiles 3986 / 3907.
-    const bool few = n_tiles <= 4096;
+    // few waves: fewer resident blocks with more registers shorten the longest lists' chains; many waves:
+    // the most blocks that fit.  The lines are in blocks (four to a 16x16 tile, one to an 8x8).  One-group
+    // times with 14 against 16 blocks an SM, us: 28,800 blocks 123 / 129, 38,400 145 / 141, 76,800 289 / 281 (tiles of
+    // 8x8: 19,200 98 / 107, 38,400 172 / 176, 57,600 256 / 254); with randomisation 38,400 152 / 168, 57,600 229 / 227;
+    // with checkpoints (60 bytes of spills at 16) 38,400 147 / 178, 76,800 295 / 305, 153,600 625 / 614.
+    const int bpt = (P.tile_w * P.tile_h) / (32 * kCompWarps);
+    const bool few = (int64_t)n_tiles * bpt <= (with_ck ? 98304 : P.aug ? 49152 : 32768);
     auto* kern = with_ck ? (work ? k_composite<true, false, true, 16> : few ? k_composite<false, false, true, 14>
                                                                            : k_composite<false, false, true, 16>)
                  : work  ? (P.aug ? k_composite<true, true, false, 16> : k_composite<true, false, false, 16>)
                  : few   ? (P.aug ? k_composite<false, true, false, 14> : k_composite<false, false, false, 14>)
                          : (P.aug ? k_composite<false, true, false, 16> : k_composite<false, false, false, 16>);
-    const int bpt = (P.tile_w * P.tile_h) / (32 * kCompWarps);
     kern<<<n_tiles * bpt, kCompWarps * 32, 0, L.stream>>>(views, v0, n_group_views, ranges, keys, vals, records, P,
                                                           out_rgb, out_depth, out_alpha, work, tile_order, ck);
     ++*L.launches;
