@@ -43,9 +43,10 @@ BWD_OPS_PER_PAIR = 50
 # the culled instances' tests and the tile-row runs of emission are left out, so their
 # fractions are lower bounds.
 PROJ_OPS, SH3_OPS, CULL_OPS = 200, 90, 35
-# The projection adjoint moves per visible instance: 40 B of partials, 236 B of FP32 attributes
-# read, 236 B of attribute gradients accumulated and 8 B of identity.
-PROJECT_BWD_BYTES = 40 + 236 + 236 + 8
+# The projection adjoint moves per visible instance: 48 B of accumulators (ten partials in three
+# 16-byte quads), 236 B of FP32 attributes read, 236 B of attribute gradients accumulated and 8 B of
+# identity.
+PROJECT_BWD_BYTES = 48 + 236 + 236 + 8
 # DRAM bytes (read + write) per launch on the full workload, from a one-pass ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum) of the full launch: 1043.7 + 756.3 MB.  Set to
 # None whenever the kernel changes after its capture.
@@ -923,7 +924,8 @@ def main():
                                 "ops_per_pair": OPS_PER_PAIR}},
         "sort": {**hbm(sort_bytes, per_step["sort"]),
                  "units": {"instances": NV, "pairs": P, "depth_passes": 4, "view_passes": vpasses,
-                           "view_key": "packed in the values" if packed else "gathered",
+                           "view_key": ("none" if vbits == 0 else "in the depth key" if vpasses == 0 else
+                                        "packed in the values" if packed else "gathered"),
                            "tile_passes": passes, "bytes_per_instance": depth_b + 12 + 64,
                            "bytes_per_pair": 8 + 4 + passes * 16}},
         "emit": {**alu(NV * (PROJ_OPS + SH3_OPS), per_step["emit"]),
@@ -945,8 +947,8 @@ def main():
         kernels["composite_bwd"] = {**alu(fw["pairs_composited"] * BWD_OPS_PER_PAIR, fk["bwd_backward"]),
                                     "units": {"pairs_composited": fw["pairs_composited"],
                                               "ops_per_pair": BWD_OPS_PER_PAIR,
-                                              "reductions": fw["bwd_reductions"],
-                                              "reductions_per_s": fw["bwd_reductions"] / (fk["bwd_backward"] / 1e3),
+                                              "partials_added": fw["bwd_reductions"],
+                                              "partials_added_per_s": fw["bwd_reductions"] / (fk["bwd_backward"] / 1e3),
                                               "workload": "800x800 view, 500k Gaussians"}}
         kernels["project_bwd"] = {**hbm(fw["visible"] * PROJECT_BWD_BYTES, fk["bwd_backward_project"]),
                                   "units": {"visible": fw["visible"], "bytes_per_visible": PROJECT_BWD_BYTES,

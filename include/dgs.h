@@ -167,8 +167,9 @@ typedef struct dgs_stats {
     int64_t px_composited;      /* pairs composited */
     int32_t path;               /* dgs_path: how the call ran */
     int32_t graph_captures;     /* graphs captured by this context so far */
-    int64_t bwd_reductions;     /* dgs_render_backward with profile = 2: global atomic adds of the
-                                   compositing adjoint's per-instance partials */
+    int64_t bwd_reductions;     /* dgs_render_backward with profile = 2: per-instance partials that the
+                                   compositing adjoint added to memory (ten per record and sub-tile,
+                                   in three vector reductions of up to four) */
 } dgs_stats;
 
 /* dgs_stats.path */
@@ -262,7 +263,7 @@ int dgs_workspace_query_batch(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nod
  * views, resolutions, node sizes, storage types and env node tables, the same node_poses and
  * output pointers, and a workspace that has not moved -- upload the host tables (camera
  * poses, intrinsics and node attribute pointers may change) and replay the graph.  Node poses
- * are read from node_poses at replay time.  If a replay finds more instances or pairs than its
+ * are read from node_poses at replay time.  Any other batch renders eagerly and is captured.  If a replay finds more instances or pairs than its
  * capacity, its kernels skip their work, the call renders again eagerly (correct outputs) and
  * recaptures with larger capacities; dgs_stats.path says which happened.  The graph keeps the
  * one or two view groups of the render it was captured from (two groups run on two streams,

@@ -46,13 +46,18 @@ __global__ void __launch_bounds__(kTsdfThreads) k_tsdf_depth(const __grid_consta
         const int mid = (lo + hi + 1) >> 1;
         if (view_of<BY_VALUE>(set, table, mid).q0 <= first) lo = mid; else hi = mid - 1;
     }
+    // most blocks lie inside one view
+    const bool whole = lo + 1 >= V || view_of<BY_VALUE>(set, table, lo + 1).q0 >= first + kTsdfThreads * kDepthItems;
+    int64_t shift = view_of<BY_VALUE>(set, table, lo).pix_off - view_of<BY_VALUE>(set, table, lo).q0;
     float a[kDepthItems], d[kDepthItems];               // loads in flight together
 #pragma unroll
     for (int m = 0; m < kDepthItems; ++m) {
         const int64_t q = first + m * kTsdfThreads + threadIdx.x;
-        while (lo + 1 < V && view_of<BY_VALUE>(set, table, lo + 1).q0 <= q) ++lo;
-        const TsdfView& cv = view_of<BY_VALUE>(set, table, lo);
-        const int64_t p = cv.pix_off + (q - cv.q0);
+        if (!whole) {
+            while (lo + 1 < V && view_of<BY_VALUE>(set, table, lo + 1).q0 <= q) ++lo;
+            shift = view_of<BY_VALUE>(set, table, lo).pix_off - view_of<BY_VALUE>(set, table, lo).q0;
+        }
+        const int64_t p = q + shift;
         a[m] = q < n_pix ? alpha[p] : 0.f;
         d[m] = q < n_pix ? depth[p] : 0.f;
     }
