@@ -120,10 +120,9 @@ typedef struct dgs_options {
                                    status of their second partition (of 4096 entries, of 3072
                                    instances) unpublished, so the waits of those behind it run out
                                    (DGS_ERR_TIMEOUT after about spin_limit_us per wave of resident
-                                   blocks); 2: with
-                                   check_binning, the host copy of the first view group's tile keys is
-                                   corrupted (two adjacent pairs of different tiles exchanged) before
-                                   the check, which must then report it; 3 (DGS_DEBUG builds only,
+                                   blocks); 2: with check_binning, the host copy of the first view
+                                   group's tile keys is corrupted (two adjacent pairs of different
+                                   tiles exchanged) before the check, which must then report it; 3 (DGS_DEBUG builds only,
                                    DGS_ERR_INVALID_ARG otherwise): the compositors of an eager render
                                    or backward are told that every view group holds half the records
                                    it does, so the bounds check on tile-list entries fails
@@ -263,8 +262,9 @@ int dgs_workspace_query_batch(dgs_ctx* ctx, const dgs_node* nodes, int32_t n_nod
  * views, resolutions, node sizes, storage types and env node tables, the same node_poses and
  * output pointers, and a workspace that has not moved -- upload the host tables (camera
  * poses, intrinsics and node attribute pointers may change) and replay the graph.  Node poses
- * are read from node_poses at replay time.  Any other batch renders eagerly and is captured.  If a replay finds more instances or pairs than its
- * capacity, its kernels skip their work, the call renders again eagerly (correct outputs) and
+ * are read from node_poses at replay time.  Any other batch renders eagerly and is captured.  If a
+ * replay finds more instances or pairs than its capacity, its kernels skip their work, the call
+ * renders again eagerly (correct outputs) and
  * recaptures with larger capacities; dgs_stats.path says which happened.  The graph keeps the
  * one or two view groups of the render it was captured from (two groups run on two streams,
  * see views_per_group); a batch that needs more groups is not captured and runs eagerly.
